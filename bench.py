@@ -853,7 +853,7 @@ def main():
     ap.add_argument("--no-cpu-all-cores", action="store_true",
                     help="skip the oracle timing over all host cores (one forked worker per core)")
     ap.add_argument("--no-fp64", action="store_true", help="skip the FP64 comparator run")
-    ap.add_argument("--plane", choices=["default", "cta", "cluster", "lines"], default="default",
+    ap.add_argument("--plane", choices=["default", "cta", "cluster", "lines", "split"], default="default",
                     help="plane-stage kernel (default: autotuned among those the grid supports)")
     ap.add_argument("--helm", choices=["default", "simt", "tc", "persist", "fused", "fused_d2v", "fused_eo", "fused_eo_ff", "simt_eo"], default="default",
                     help="per-wavenumber stage of the mixed path (default: the fused stage where the group "

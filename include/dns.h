@@ -145,12 +145,15 @@ typedef struct {
                                       against 1 and 3 only up to My = 49 (linear groups at every
                                       size); 1 and 3 are timed against each other at every size */
     int plane;                     /* plane stage: 0 autotuned where several kernels exist (else
-                                      the only one; FP64 defaults to 1), 1 one CTA per plane
+                                      the only one; 5 for FP64 and for 128-point grids where the
+                                      size has it), 1 one CTA per plane
                                       (sizes <= 64), 2 a thread-block cluster per plane (64x64
                                       single precision, and every size with a 128), 3 one CTA
                                       per plane with each 1-D transform owned by one group of
-                                      threads (mixed precision, sizes <= 64); a request for a
-                                      variant the group's size lacks is ignored */
+                                      threads (mixed precision, sizes <= 64), 5 three launches
+                                      (z, x, z) that hand the planes on through L2 (both
+                                      precisions, sizes >= 32); a request for a variant the
+                                      group's size lacks is ignored */
     int helm;                      /* mixed path per-wavenumber stage: 0 autotuned at
                                       dns_bind_workspace (DNS groups: 1, 2 and 8, each timed with
                                       the y-derivatives and the forcing, against 4 to 7; linear
@@ -325,7 +328,8 @@ const char* dns_last_error(const dns_handle* h);
  * dns_bind_workspace): ygemm 1 register-tiled FP32 / 2 tcgen05 y-contraction /
  * 3 register-tiled FP32 in parity blocks;
  * plane 1 one CTA per plane / 2 a thread-block cluster per plane / 3 line-owned
- * single CTA per plane; helm 1 register-tiled FP32 / 2 tcgen05 implicit apply /
+ * single CTA per plane / 5 three launches per plane stage (4 the linear groups'
+ * own); helm 1 register-tiled FP32 / 2 tcgen05 implicit apply /
  * 3 persistent register-tiled FP32 / 4 the fused per-wavenumber stage / 5 the
  * fused stage with D2 v inside it / 6 the fused stage in parity blocks / 7 the
  * same with its float-float D2 v / 8 the register-tiled FP32 stage with its

@@ -314,7 +314,7 @@ _PRECS = {"fp64": DNS_PREC_FP64, "mixed": DNS_PREC_MIXED}
 _YGEMM = {"default": 0, "auto": 0, "simt": 1, "tc": 2, "simt_eo": 3}
 
 
-_PLANE = {"default": 0, "auto": 0, "cta": 1, "cluster": 2, "lines": 3}
+_PLANE = {"default": 0, "auto": 0, "cta": 1, "cluster": 2, "lines": 3, "split": 5}
 
 
 _HELM = {"default": 0, "auto": 0, "simt": 1, "tc": 2, "persist": 3, "fused": 4, "fused_d2v": 5, "fused_eo": 6, "fused_eo_ff": 7, "simt_eo": 8}
@@ -339,7 +339,7 @@ def make_config(groups, precision="fp64", use_graph=False, ygemm="default", auto
     time (None: the DNS_AUTOTUNE_CACHE environment variable, if set).
     ygemm, plane, helm: kernel-variant requests of the mixed path ("default":
     autotuned at bind time; dns_config in include/dns.h describes each):
-    ygemm simt | tc | simt_eo; plane cta | cluster | lines; helm simt | tc |
+    ygemm simt | tc | simt_eo; plane cta | cluster | lines | split; helm simt | tc |
     persist | fused | fused_d2v | fused_eo | fused_eo_ff | simt_eo."""
     arr = (dns_group_desc * len(groups))()
     for i, g in enumerate(groups):

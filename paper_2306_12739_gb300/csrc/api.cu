@@ -274,6 +274,10 @@ size_t layout_group(dns_handle* h, HostGroup& G, size_t cur) {
     const size_t elem = precision_mixed(h) ? sizeof(float2) : sizeof(double2);
     add(&v.P5, elem * 5 * S);
     add(&v.N3, elem * 3 * S);
+    if (v.plane == 5) {
+        add(&v.COL, dnsk::plane_split_col_bytes(v, !precision_mixed(h)));
+        add((void**)&v.psum, dnsk::plane_split_psum_bytes(v));
+    }
     if (precision_mixed(h)) add((void**)&v.P5d, sizeof(double2) * 5 * S);
     add((void**)&v.st_y, sizeof(double) * (size_t)v.E * v.ny * 6);
     add((void**)&v.st_out, sizeof(double) * (size_t)v.E * 9);
@@ -345,6 +349,15 @@ struct Timer {
     std::vector<int> cls;
 };
 
+// one of the mixed plane-stage kernels
+void launch_plane_mixed(const GroupView& g, int variant, const double* U, const double* W, cudaStream_t st) {
+    if (variant == 5) dnsk::launch_plane_split(g, false, U, W, st);
+    else if (variant == 2) dnsk::launch_plane_cl(g, false, U, W, st);
+    else if (variant == 3) dnsk::launch_plane_lines(g, U, W, st);
+    else dnsk::launch_plane_f32(g, U, W, st);
+}
+int plane_launches(const GroupView& g) { return g.plane == 5 ? 3 : 1; }
+
 void enqueue_group(dns_handle* h, HostGroup& G, cudaStream_t st, Timer* tm) {
     auto mark = [&](int c) {
         if (!tm) return;
@@ -375,10 +388,9 @@ void enqueue_group(dns_handle* h, HostGroup& G, cudaStream_t st, Timer* tm) {
         if (precision_mixed(h) && g.helm == 4) {
             // the derivatives of this sub-step's state came with the previous
             // fused launch (or with the setting of the state)
-            if (g.plane == 2) dnsk::launch_plane_cl(g, false, cU, cW, st);
-            else if (g.plane == 3) dnsk::launch_plane_lines(g, cU, cW, st);
-            else dnsk::launch_plane_f32(g, cU, cW, st);
+            launch_plane_mixed(g, g.plane, cU, cW, st);
             mark(DNS_K_PLANE);
+            h->launches += plane_launches(g) - 1;
             if (g.shared_mean && g.E > 1) { dnsk::launch_shared_mean(g, false, st); h->launches += 1; }
             if (s == 0 && g.fn > 0 && !side_noise) { dnsk::launch_stoch_noise(g, st); h->launches += 1; }
             if (s == 0 && side_noise) cudaStreamWaitEvent(st, G.njoin, 0);
@@ -398,10 +410,9 @@ void enqueue_group(dns_handle* h, HostGroup& G, cudaStream_t st, Timer* tm) {
             else dnsk::launch_yderiv_t(g, cv, ce, st, sprev);
             mark(DNS_K_YDERIV);
             if (g.lin) dnsk::launch_lin_plane(g, false, st);
-            else if (g.plane == 2) dnsk::launch_plane_cl(g, false, cU, cW, st);
-            else if (g.plane == 3) dnsk::launch_plane_lines(g, cU, cW, st);
-            else dnsk::launch_plane_f32(g, cU, cW, st);
+            else launch_plane_mixed(g, g.plane, cU, cW, st);
             mark(DNS_K_PLANE);
+            h->launches += plane_launches(g) - 1;
             if (g.shared_mean && g.E > 1) { dnsk::launch_shared_mean(g, false, st); h->launches += 1; }
             if (s == 0 && g.fn > 0 && !side_noise) { dnsk::launch_stoch_noise(g, st); h->launches += 1; }
             if (s == 0 && side_noise) cudaStreamWaitEvent(st, G.njoin, 0);
@@ -411,9 +422,11 @@ void enqueue_group(dns_handle* h, HostGroup& G, cudaStream_t st, Timer* tm) {
             dnsk::launch_yderiv<double>(g, cv, ce, g.P5, st, sprev);
             mark(DNS_K_YDERIV);
             if (g.lin) dnsk::launch_lin_plane(g, true, st);
+            else if (g.plane == 5) dnsk::launch_plane_split(g, true, cU, cW, st);
             else if (g.plane == 2) dnsk::launch_plane_cl(g, true, cU, cW, st);
             else dnsk::launch_plane_state<double>(g, cU, cW, st);
             mark(DNS_K_PLANE);
+            h->launches += plane_launches(g) - 1;
             if (g.shared_mean && g.E > 1) { dnsk::launch_shared_mean(g, true, st); h->launches += 1; }
             if (s == 0 && g.fn > 0 && !side_noise) { dnsk::launch_stoch_noise(g, st); h->launches += 1; }
             if (s == 0 && side_noise) cudaStreamWaitEvent(st, G.njoin, 0);
@@ -473,7 +486,8 @@ std::string tune_key(const GroupView& v) {
 }
 
 // plane-stage variants: 1 one CTA per plane, 2 a thread-block cluster per
-// plane, 3 line-owned single CTA (single precision only)
+// plane, 3 line-owned single CTA (single precision only); 5, three launches,
+// goes by plane_split_supported
 bool plane_variant_ok(bool mixed, const GroupView& v, int c) {
     const size_t lim = 227 * 1024;
     // the rotational form exists in the line-owned kernel (single precision) and
@@ -493,6 +507,15 @@ bool plane_variant_ok(bool mixed, const GroupView& v, int c) {
     }
     return false;
 }
+
+// Where the plane stage runs as three launches (k_plane_split.cu) unless another
+// kernel is asked for:
+//   128-point grids, where a plane does not fit one SM: 404 -> 153 us a launch
+//   against the cluster kernel on 128x97x128 x 4, 1099 -> 670 us in FP64;
+//   FP64 everywhere it can (grids of 32 points up): 991 -> 548 us on 64x65x64 x
+//   4, 154 -> 144 on 32x33x32 x 2; the single-CTA kernel spends its FP64 pipe on
+//   radix-2 to 4 passes and leaves SMs idle at few planes.
+bool plane_split_default(const GroupView& v, bool mixed) { return !mixed || v.mx == 128 || v.mz == 128; }
 
 std::string tune_helm_key(const GroupView& v) {
     char b[128];
@@ -644,6 +667,9 @@ int choose_variants(dns_handle* h, const dns_config* cfg, GroupView& v, int gi) 
             return fail(h, DNS_ERR_UNSUPPORTED, "group %d: no plane-stage kernel for %dx%d", gi, d.mx, d.mz);
         v.plane = navail == 1 ? (ok[1] ? 1 : ok[2] ? 2 : 3) : (mixed ? 0 : 1);
         if (navail > 1 && cfg->plane >= 1 && cfg->plane <= 3 && ok[cfg->plane]) v.plane = cfg->plane;
+        if (dnsk::plane_split_supported(v) && (cfg->plane == 5 || (!(cfg->plane >= 1 && cfg->plane <= 3 && ok[cfg->plane]) &&
+                                                                   plane_split_default(v, mixed))))
+            v.plane = 5;
     }
     if (precision_mixed(h)) {
         size_t m1 = dnsk::helm_t_smem_bytes(v), m2 = dnsk::yderiv_t_smem_bytes(v), m3 = dnsk::forcing_t_smem_bytes(v);
@@ -934,6 +960,7 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
     dnsk::set_attributes_yderiv_tc();
     dnsk::set_attributes_plane_cl();
     dnsk::set_attributes_plane_lines();
+    dnsk::set_attributes_plane_split();
     dnsk::set_attributes_helm_tc();
     dnsk::set_attributes_linear();
     dnsk::set_attributes_spec();
@@ -1015,9 +1042,7 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
             for (int cand = 1; cand <= 3; ++cand) {
                 if (!plane_variant_ok(true, v, cand)) continue;
                 auto run = [&]() {
-                    if (cand == 2) dnsk::launch_plane_cl(v, false, v.U_t, v.W_t, st);
-                    else if (cand == 3) dnsk::launch_plane_lines(v, v.U_t, v.W_t, st);
-                    else dnsk::launch_plane_f32(v, v.U_t, v.W_t, st);
+                    launch_plane_mixed(v, cand, v.U_t, v.W_t, st);
                 };
                 for (int w = 0; w < 2; ++w) run();
                 cudaEventRecord(e0, st);

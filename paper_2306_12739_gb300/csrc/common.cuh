@@ -15,7 +15,7 @@ namespace dnsk {
 constexpr int BOUNDS_FLAG = 0x40000000;
 enum CheckKernel {
     CK_SELFTEST = 1, CK_SPEC = 2, CK_D2V = 3, CK_PLANE_LINES = 4, CK_YDERIV_T = 5, CK_FORCING_T = 6,
-    CK_HELM_T = 7, CK_PACK = 8, CK_UNPACK = 9, CK_SPEC_SMEM = 10
+    CK_HELM_T = 7, CK_PACK = 8, CK_UNPACK = 9, CK_SPEC_SMEM = 10, CK_PLANE_SPLIT = 11
 };
 __device__ __forceinline__ bool ck_record(int* status, bool ok, int kernel, long long index) {
     if (!ok) atomicCAS(status, 0, BOUNDS_FLAG | (kernel << 24) | (int)(index & 0xFFFFFF));

@@ -22,7 +22,7 @@ struct GroupView {
     int ygemm;            // mixed path y-derivatives: 1 register-tiled FP32, 2 tcgen05 split-BF16,
                           // 3 register-tiled FP32 in parity blocks; 0 = autotune
     int plane;            // plane stage: 1 single-CTA kernel, 2 cluster kernel, 3 line-owned
-                          // single-CTA kernel (mixed path); 0 = autotune
+                          // single-CTA kernel (mixed path), 5 the three-launch split one; 0 = autotune
     const void* Atc;      // tensor-core A image: [D1_int; D2_int] in 3 BF16 pieces
     int helm;             // mixed path implicit apply: 1 register-tiled FP32, 2 tcgen05, 3 persistent
                           // register-tiled FP32 with double-buffered operator copies, 4 the fused
@@ -103,6 +103,8 @@ struct GroupView {
     // P layout work arrays (element type by precision)
     void* P5;    // 5 fields: v, Dv, D2v, eta, Deta
     void* N3;    // 3 fields: Nu, Nv, Nw
+    void* COL;     // split plane stage: columns between its launches [Ny E][9 or 6 fields][Mz][row] (k_plane_split.cu)
+    double2* psum; // its partial sums of u v, w v
     double2* P5d;  // FP64 copy for statistics (== P5 in FP64 mode)
     // statistics
     double* st_y;    // [E][Ny][6]: uu, vv, ww, uv, maxdiv, nonfinite
@@ -213,6 +215,12 @@ void set_attributes_plane_f32();
 bool launch_plane_lines(const GroupView& g, const double* U, const double* W, cudaStream_t st);
 size_t plane_lines_smem_bytes(int mx, int mz);
 void set_attributes_plane_lines();
+// the plane stage as z-inverse, x and z-forward launches (k_plane_split.cu)
+bool plane_split_supported(const GroupView& g);
+size_t plane_split_col_bytes(const GroupView& g, bool fp64);
+size_t plane_split_psum_bytes(const GroupView& g);
+void launch_plane_split(const GroupView& g, bool fp64, const double* U, const double* W, cudaStream_t st);
+void set_attributes_plane_split();
 int plane_threads();
 
 }  // namespace dnsk
