@@ -40,6 +40,7 @@ struct HostGroup {
     dnsb::GridOps grid;
     dnsb::CnOps ops[2];
     std::vector<double> kxt, kzt, k2t, k2inv, twx, twz, opsdev[2], mopsdev[2], D1i, D2i;
+    std::vector<double> ops64[2], D1EO64, D2EO64;   // FP64 path: the operators in parity blocks
     std::vector<float> kxtf, kztf, k2invf, twxf, twzf, opsf[2], opsfT[2], D1T, D2T, D2Tl, opsEO[2], D1EO, D2EO, D2lEO;
     std::vector<uint16_t> Atc, Htc[2], D2oz;
     std::vector<int> D2ozexp;
@@ -204,6 +205,24 @@ void build_eo_images(HostGroup& G, bool ops) {
     dnsk::spec_eo_image(G.D2i.data(), v.ny, false, G.D2lEO.data(), true);
 }
 
+// The FP64 parity-block images: D1, D2 (every group: the statistics use them)
+// and, on the FP64 path, M and P of every pair, which replace the full
+// matrices G.opsdev.
+void build_eo64_images(HostGroup& G, bool ops) {
+    const GroupView& v = G.v;
+    const size_t nn = (size_t)v.ny * v.ny, mat = dnsk::spec_eo_mat_floats(v.ny);
+    for (int hi = 0; hi < 2 && ops; ++hi) {
+        G.ops64[hi].resize((size_t)v.npairs * 4 * mat);
+        for (size_t blk = 0; blk < (size_t)v.npairs * 4; ++blk)
+            dnsk::spec_eo_image64(&G.opsdev[hi][blk * nn], v.ny, false, &G.ops64[hi][blk * mat]);
+        std::vector<double>().swap(G.opsdev[hi]);
+    }
+    G.D1EO64.resize(mat);
+    G.D2EO64.resize(mat);
+    dnsk::spec_eo_image64(G.D1i.data(), v.ny, true, G.D1EO64.data());
+    dnsk::spec_eo_image64(G.D2i.data(), v.ny, false, G.D2EO64.data());
+}
+
 size_t layout_group(dns_handle* h, HostGroup& G, size_t cur) {
     GroupView& v = G.v;
     G.slots.clear();
@@ -216,7 +235,8 @@ size_t layout_group(dns_handle* h, HostGroup& G, size_t cur) {
     const size_t nn = (size_t)v.ny * v.ny;
     add((void**)&v.D1, sizeof(double) * v.my * v.my);
     add((void**)&v.D1i, sizeof(double) * nn);
-    add((void**)&v.D2i, sizeof(double) * nn);
+    add((void**)&v.D1EO64, sizeof(double) * dnsk::spec_eo_mat_floats(v.ny));
+    add((void**)&v.D2EO64, sizeof(double) * dnsk::spec_eo_mat_floats(v.ny));
     add((void**)&v.D1T, sizeof(float) * (size_t)v.ny * v.rp);
     add((void**)&v.D2T, sizeof(float) * (size_t)v.ny * v.rp);
     add((void**)&v.D2Tl, sizeof(float) * (size_t)v.ny * v.rp);
@@ -244,7 +264,8 @@ size_t layout_group(dns_handle* h, HostGroup& G, size_t cur) {
     add((void**)&v.kztf, sizeof(float) * v.nkz);
     add((void**)&v.k2invf, sizeof(float) * v.nmodes);
     for (int hi = 0; hi < 2; ++hi) {
-        add((void**)&v.ops[hi], sizeof(double) * (size_t)v.npairs * 4 * nn);
+        if (!precision_mixed(h))
+            add((void**)&v.ops64[hi], sizeof(double) * (size_t)v.npairs * 4 * dnsk::spec_eo_mat_floats(v.ny));
         if (precision_mixed(h)) {
             add((void**)&v.opsfT[hi], sizeof(float) * (size_t)v.npairs * 4 * v.ny * v.rp);
             if (helm_tc_candidate(v)) add((void**)&v.Htc[hi], (size_t)v.npairs * 2 * 3 * 64 * 2 * v.kp * sizeof(uint16_t));
@@ -419,7 +440,7 @@ void enqueue_group(dns_handle* h, HostGroup& G, cudaStream_t st, Timer* tm) {
             if (g.helm == 1 && g.step_eo) dnsk::launch_forcing_eo(g, s, st);
             else dnsk::launch_forcing_t(g, s, st);
         } else {
-            dnsk::launch_yderiv<double>(g, cv, ce, g.P5, st, sprev);
+            dnsk::launch_yderiv64(g, cv, ce, (double2*)g.P5, st, sprev);
             mark(DNS_K_YDERIV);
             if (g.lin) dnsk::launch_lin_plane(g, true, st);
             else if (g.plane == 5) dnsk::launch_plane_split(g, true, cU, cW, st);
@@ -430,7 +451,7 @@ void enqueue_group(dns_handle* h, HostGroup& G, cudaStream_t st, Timer* tm) {
             if (g.shared_mean && g.E > 1) { dnsk::launch_shared_mean(g, true, st); h->launches += 1; }
             if (s == 0 && g.fn > 0 && !side_noise) { dnsk::launch_stoch_noise(g, st); h->launches += 1; }
             if (s == 0 && side_noise) cudaStreamWaitEvent(st, G.njoin, 0);
-            dnsk::launch_forcing<double>(g, s, st);
+            dnsk::launch_forcing64(g, s, st);
         }
         mark(DNS_K_FORCING);
         // per-wavenumber implicit apply (and the rows of the mean-flow update)
@@ -440,7 +461,7 @@ void enqueue_group(dns_handle* h, HostGroup& G, cudaStream_t st, Timer* tm) {
             else if (g.step_eo) dnsk::launch_helm_eo(g, s, st);
             else dnsk::launch_helm_t(g, s, st);
         } else {
-            dnsk::launch_helm(g, s, st);
+            dnsk::launch_helm64(g, s, st);
         }
         mark(DNS_K_HELM);
         if (g.lin) {   // no mean flow
@@ -901,6 +922,7 @@ int dns_create(const dns_config* cfg, void* cuda_stream, dns_handle** out) {
         if (precision_mixed(h) && (eo_images(v) || ygemm_eo_candidate(v))) build_eo_images(G, eo_images(v));
         if (precision_mixed(h) && helm_tc_candidate(v))
             for (int hi = 0; hi < 2; ++hi) G.Htc[hi] = dnsk::helm_tc_a_images(G.opsdev[hi], v.npairs, v.ny, v.kp);
+        build_eo64_images(G, !precision_mixed(h));
         if (!lin) G.twx = dnsb::twiddles(d.mx);
         G.twz = dnsb::twiddles(d.mz);
         G.twxf.assign(G.twx.begin(), G.twx.end());
@@ -965,6 +987,7 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
     dnsk::set_attributes_linear();
     dnsk::set_attributes_spec();
     dnsk::set_attributes_step_eo();
+    dnsk::set_attributes_step64();
     dnsk::set_attributes_d2v_tc();
     {
         int rc0 = check(h, cudaGetLastError(), "kernel attributes");
@@ -983,7 +1006,8 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
         const Up ups[] = {
             {v.D1, G.grid.D1.data(), G.grid.D1.size() * 8},
             {v.D1i, G.D1i.data(), G.D1i.size() * 8},
-            {v.D2i, G.D2i.data(), G.D2i.size() * 8},
+            {v.D1EO64, G.D1EO64.data(), G.D1EO64.size() * 8},
+            {v.D2EO64, G.D2EO64.data(), G.D2EO64.size() * 8},
             {v.ccw, G.grid.ccw.data(), G.grid.ccw.size() * 8},
             {v.kxt, G.kxt.data(), G.kxt.size() * 8},
             {v.kzt, G.kzt.data(), G.kzt.size() * 8},
@@ -996,8 +1020,8 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
             {v.kxtf, G.kxtf.data(), G.kxtf.size() * 4},
             {v.kztf, G.kztf.data(), G.kztf.size() * 4},
             {v.k2invf, G.k2invf.data(), G.k2invf.size() * 4},
-            {v.ops[0], G.opsdev[0].data(), G.opsdev[0].size() * 8},
-            {v.ops[1], G.opsdev[1].data(), G.opsdev[1].size() * 8},
+            {v.ops64[0], G.ops64[0].data(), G.ops64[0].size() * 8},
+            {v.ops64[1], G.ops64[1].data(), G.ops64[1].size() * 8},
             {v.opsfT[0], G.opsfT[0].data(), G.opsfT[0].size() * 4},
             {v.opsfT[1], G.opsfT[1].data(), G.opsfT[1].size() * 4},
             {v.D1T, G.D1T.data(), G.D1T.size() * 4},

@@ -54,7 +54,8 @@ struct GroupView {
     // constants
     const double* D1;     // [My][My]
     const double* D1i;    // [Ny][Ny]
-    const double* D2i;    // [Ny][Ny]
+    const double* D1EO64; // D1, D2 (interior) in parity blocks
+    const double* D2EO64;
     const float* D1T;     // mixed path, transposed and row-padded: D1T[k][r] = D1i[r][k], [Ny][rp]
     const float* D2T;
     const float* D2Tl;    // D2T's residual: D2i - (double) D2T in single precision (compensated D2 v)
@@ -86,7 +87,8 @@ struct GroupView {
     const float* kxtf;
     const float* kztf;
     const float* k2invf;
-    const double* ops[2];   // per h index: [npairs][4][Ny][Ny]  (Mv, Pv, Me, Pe)
+    const double* ops64[2]; // FP64 path, per h index: [npairs][4] matrices (Mv, Pv, Me, Pe) in parity
+                            // blocks (eo.cuh), each eo_mat(Ny) doubles
     const float* opsfT[2];  // mixed path, per h index: [npairs][4][Ny][rp], transposed and row-padded
                             // single-precision (Mv - I), Pv, (Me - I), Pe
     const double* mops[2];  // per h index: MU [Ny][Ny], PU [Ny][Ny], bU [Ny][2], Ug [Ny], PD [Ny][My]
@@ -115,17 +117,18 @@ struct GroupView {
 };
 
 // sprev >= 0: the launch also carries the mean-flow finish of sub-step sprev
-template <typename T>
-void launch_yderiv(const GroupView& g, const double2* v, const double2* e, void* P5, cudaStream_t st, int sprev = -1);
+void launch_yderiv64(const GroupView& g, const double2* v, const double2* e, double2* P5, cudaStream_t st,
+                     int sprev = -1);
+void launch_forcing64(const GroupView& g, int s, cudaStream_t st);
+void launch_helm64(const GroupView& g, int s, cudaStream_t st);
+cudaError_t load_yderiv64();   // loads k_yderiv64 (the statistics run it)
+void set_attributes_step64();
 template <typename T>
 void launch_plane_state(const GroupView& g, const double* U, const double* W, cudaStream_t st);
-template <typename T>
-void launch_forcing(const GroupView& g, int s, cudaStream_t st);
-void launch_helm(const GroupView& g, int s, cudaStream_t st);
 void launch_mean_finish(const GroupView& g, int s, cudaStream_t st);
 // CTAs of the mean-flow rows carried by the implicit-apply launches (8 rows each)
 __host__ __device__ inline int mean_row_ctas(const GroupView& g) { return g.lin ? 0 : g.E * ((g.ny + 7) / 8); }
-// Members per CTA of the implicit-apply kernels (k_helm, k_helm_t).  A DNS
+// Members per CTA of the implicit-apply kernels (k_helm64 takes at most 8).  A DNS
 // group has hundreds of wavenumber pairs and keeps all its members in one CTA
 // (operator reuse); a linear group has only Kz + 1 pairs, so its members are
 // split into chunks until one group alone gives about one CTA per SM.
@@ -185,6 +188,7 @@ void launch_eo_derivs(const GroupView& g, cudaStream_t st);
 // one Ny x Ny row-major matrix (centro-symmetric, or anti-centro-symmetric when
 // anti) as its two parity blocks, transposed and row-padded (out: spec_eo_mat_floats)
 void spec_eo_image(const double* A, int ny, bool anti, float* out, bool residual = false);
+void spec_eo_image64(const double* A, int ny, bool anti, double* out);
 size_t spec_smem_bytes(const GroupView& g);
 void launch_spec(const GroupView& g, int s, cudaStream_t st);
 void set_attributes_spec();

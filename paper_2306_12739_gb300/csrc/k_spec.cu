@@ -1358,28 +1358,37 @@ void launch_eo_derivs(const GroupView& g, cudaStream_t st) {
 // rows from the even part, Aoe[i][k] = A[i][k] + A[i][R k], 2 A[i][c] (k = c).
 // Each block transposed [k][row], rows padded to RP2: the even output rows'
 // block first (KE inputs), then the odd output rows' block.
-void spec_eo_image(const double* A, int ny, bool anti, float* out, bool residual) {
+template <typename Put>
+static void eo_blocks(const double* A, int ny, bool anti, Put put) {
     const int NE = spc::eo_ne(ny), NO = ny / 2, RP2 = spc::eo_rp(ny);
-    const size_t mat = spc::eo_mat(ny);
-    for (size_t i = 0; i < mat; ++i) out[i] = 0.f;
     auto a = [&](int i, int j) { return A[(size_t)i * ny + j]; };
     const int KE = anti ? NO : NE, KO = anti ? NE : NO;
-    float* be = out;
-    float* bo = out + (size_t)KE * RP2;
+    const size_t bo = (size_t)KE * RP2;
     for (int i = 0; i < NE; ++i)
         for (int k = 0; k < KE; ++k) {
             double v;
             if (i < NO) v = (!anti && k == NO) ? 2.0 * a(i, NO) : (anti ? a(i, k) - a(i, ny - 1 - k) : a(i, k) + a(i, ny - 1 - k));
             else v = a(NO, k);                    // the centre row (odd Ny)
-            be[(size_t)k * RP2 + i] = residual ? (float)(v - (double)(float)v) : (float)v;
+            put((size_t)k * RP2 + i, v);
         }
     for (int i = 0; i < NO; ++i)
         for (int k = 0; k < KO; ++k) {
             double v;
             if (anti) v = (k == NO) ? 2.0 * a(i, NO) : a(i, k) + a(i, ny - 1 - k);
             else v = a(i, k) - a(i, ny - 1 - k);
-            bo[(size_t)k * RP2 + i] = residual ? (float)(v - (double)(float)v) : (float)v;
+            put(bo + (size_t)k * RP2 + i, v);
         }
+}
+
+void spec_eo_image(const double* A, int ny, bool anti, float* out, bool residual) {
+    for (size_t i = 0; i < spc::eo_mat(ny); ++i) out[i] = 0.f;
+    eo_blocks(A, ny, anti, [&](size_t i, double v) { out[i] = residual ? (float)(v - (double)(float)v) : (float)v; });
+}
+
+// the same in double (the FP64 path)
+void spec_eo_image64(const double* A, int ny, bool anti, double* out) {
+    for (size_t i = 0; i < spc::eo_mat(ny); ++i) out[i] = 0.0;
+    eo_blocks(A, ny, anti, [&](size_t i, double v) { out[i] = v; });
 }
 
 // the shapes with their own instantiation: (Ny, members per chunk)

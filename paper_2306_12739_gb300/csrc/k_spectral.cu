@@ -1,10 +1,4 @@
 // Spectral-space kernels of one CN/RK3 sub-step (paper Sec. 3):
-//   k_yderiv      Dv, D2v, D eta on the interior nodes (y-contraction with the
-//                 shared Chebyshev operators, Sec. 3.1) and the H -> P relayout
-//   k_forcing     F = -k^2 Nv - D(i kx Nu + i kz Nw), G = i kz Nu - i kx Nw
-//                 (Eqs. Dv, eta) and the RK3 combination of Sec. 3.1
-//   k_helm        x_s = M_h x_t + P_h F~ per wavenumber pair (Eqs. CN1, CN2),
-//                 with M_1 x_t computed once and reused by sub-steps 2 and 3
 //   k_mean_finish U00, W00 update (Eqs. CN3, CN4): the Poiseuille constant-flux
 //                 gamma and the profiles, after the rows (mean.cuh) that run as
 //                 extra CTAs of the implicit apply
@@ -14,180 +8,6 @@
 #include "mean.cuh"
 
 namespace dnsk {
-
-// ------------------------------------------------------------------ y-derivs
-
-constexpr int QB = 8;   // modes per tile
-constexpr int EB = 4;   // members per tile
-
-// T is the arithmetic (and output) type: double for the FP64 path, float for
-// the mixed path (the FP64 state is rounded to float on load).
-template <typename T>
-__global__ void __launch_bounds__(256) k_yderiv(const double2* __restrict__ v, const double2* __restrict__ et,
-                                                const T* __restrict__ D1i, const T* __restrict__ D2i,
-                                                typename C2<T>::type* __restrict__ P5, int Ny, int E, int nmodes,
-                                                GroupView g, int sprev) {
-    typedef typename C2<T>::type C;
-    extern __shared__ __align__(16) unsigned char sm[];
-    if (mean_finish_rows(g, sprev, (E + EB - 1) / EB, sm)) return;
-    C* xv = (C*)sm;                 // [QB][Ny][EB]
-    C* xe = xv + QB * Ny * EB;
-    const int q0 = blockIdx.x * QB, e0 = blockIdx.y * EB;
-    const int tile = QB * Ny * EB;
-    for (int idx = threadIdx.x; idx < tile; idx += blockDim.x) {
-        int ee = idx % EB;
-        int y = (idx / EB) % Ny;
-        int qq = idx / (EB * Ny);
-        int q = q0 + qq, e = e0 + ee;
-        C a = czero<C>(), b = a;
-        if (q < nmodes && e < E) {
-            size_t o = ((size_t)q * Ny + y) * E + e;
-            double2 va = v[o], vb = et[o];
-            a.x = (T)va.x; a.y = (T)va.y;
-            b.x = (T)vb.x; b.y = (T)vb.y;
-        }
-        xv[idx] = a;
-        xe[idx] = b;
-    }
-    __syncthreads();
-    const size_t fs = (size_t)Ny * E * nmodes;
-    for (int idx = threadIdx.x; idx < tile; idx += blockDim.x) {
-        int qq = idx % QB;
-        int ee = (idx / QB) % EB;
-        int y = idx / (QB * EB);
-        int q = q0 + qq, e = e0 + ee;
-        T dvx = 0, dvy = 0, d2x = 0, d2y = 0, dex = 0, dey = 0;
-        const T* r1 = D1i + (size_t)y * Ny;
-        const T* r2 = D2i + (size_t)y * Ny;
-        for (int k = 0; k < Ny; ++k) {
-            T d1 = __ldg(r1 + k), d2 = __ldg(r2 + k);
-            C a = xv[(qq * Ny + k) * EB + ee];
-            C b = xe[(qq * Ny + k) * EB + ee];
-            dvx += d1 * a.x; dvy += d1 * a.y;
-            d2x += d2 * a.x; d2y += d2 * a.y;
-            dex += d1 * b.x; dey += d1 * b.y;
-        }
-        if (q < nmodes && e < E) {
-            size_t o = ((size_t)y * E + e) * nmodes + q;
-            C a = xv[(qq * Ny + y) * EB + ee];
-            C b = xe[(qq * Ny + y) * EB + ee];
-            C c;
-            P5[o] = a;
-            c.x = dvx; c.y = dvy; P5[fs + o] = c;
-            c.x = d2x; c.y = d2y; P5[2 * fs + o] = c;
-            P5[3 * fs + o] = b;
-            c.x = dex; c.y = dey; P5[4 * fs + o] = c;
-        }
-    }
-}
-
-template <typename T> __host__ __device__ const T* d1i_of(const GroupView& g);
-template <> __host__ __device__ const double* d1i_of<double>(const GroupView& g) { return g.D1i; }
-template <typename T> __host__ __device__ const T* d2i_of(const GroupView& g);
-template <> __host__ __device__ const double* d2i_of<double>(const GroupView& g) { return g.D2i; }
-
-template <typename T>
-void launch_yderiv(const GroupView& g, const double2* v, const double2* e, void* P5, cudaStream_t st, int sprev) {
-    dim3 grid((g.nmodes + QB - 1) / QB, (g.E + EB - 1) / EB);
-    grid.y += mean_finish_extra_rows(g, grid.x, sprev);
-    size_t smem = 2 * (size_t)QB * g.ny * EB * sizeof(typename C2<T>::type);
-    k_yderiv<T><<<grid, 256, smem, st>>>(v, e, d1i_of<T>(g), d2i_of<T>(g), (typename C2<T>::type*)P5, g.ny, g.E,
-                                         g.nmodes, g, sprev);
-}
-template void launch_yderiv<double>(const GroupView&, const double2*, const double2*, void*, cudaStream_t, int);
-
-// ------------------------------------------------------------------- forcing
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_forcing(GroupView g, int s) {
-    typedef typename C2<T>::type C;
-    extern __shared__ __align__(16) unsigned char sm[];
-    C* phi = (C*)sm;   // [QB][Ny][EB], i kx Nu + i kz Nw in the arithmetic type T
-    const T* D1 = d1i_of<T>(g);
-    const int Ny = g.ny, E = g.E, nmodes = g.nmodes, NKX = g.nkx;
-    const int q0 = blockIdx.x * QB, e0 = blockIdx.y * EB;
-    const int tile = QB * Ny * EB;
-    const size_t fs = (size_t)Ny * E * nmodes;
-    const C* N3 = (const C*)g.N3;
-    for (int idx = threadIdx.x; idx < tile; idx += blockDim.x) {
-        int qq = idx % QB;
-        int ee = (idx / QB) % EB;
-        int y = idx / (QB * EB);
-        int q = q0 + qq, e = e0 + ee;
-        C p = czero<C>();
-        if (q < nmodes && e < E) {
-            size_t o = ((size_t)y * E + e) * nmodes + q;
-            C nu = N3[o], nw = N3[2 * fs + o];
-            int mi = q / NKX, n = q - mi * NKX;
-            T kx = (T)g.kxt[n], kz = (T)g.kzt[mi];
-            // i kx Nu + i kz Nw
-            T ax = kx * nu.x + kz * nw.x;
-            T ay = kx * nu.y + kz * nw.y;
-            p.x = -ay; p.y = ax;
-        }
-        phi[(qq * Ny + y) * EB + ee] = p;
-    }
-    __syncthreads();
-    const int q_mean = mean_mode(g);
-    for (int idx = threadIdx.x; idx < tile; idx += blockDim.x) {
-        int ee = idx % EB;
-        int y = (idx / EB) % Ny;
-        int qq = idx / (EB * Ny);
-        int q = q0 + qq, e = e0 + ee;
-        if (q >= nmodes || e >= E) continue;
-        T tx = 0, ty = 0;
-        const T* r1 = D1 + (size_t)y * Ny;
-        for (int k = 0; k < Ny; ++k) {
-            T d = __ldg(r1 + k);
-            C p = phi[(qq * Ny + k) * EB + ee];
-            tx += d * p.x; ty += d * p.y;
-        }
-        const double sx = (double)tx, sy = (double)ty;
-        size_t o = ((size_t)y * E + e) * nmodes + q;
-        C nu = N3[o], nv = N3[fs + o], nw = N3[2 * fs + o];
-        int mi = q / NKX, n = q - mi * NKX;
-        double kx = g.kxt[n], kz = g.kzt[mi], k2 = g.k2t[q];
-        double2 F, G;
-        F.x = -k2 * (double)nv.x - sx;
-        F.y = -k2 * (double)nv.y - sy;
-        // i kz Nu - i kx Nw
-        double bx = kz * (double)nu.x - kx * (double)nw.x;
-        double by = kz * (double)nu.y - kx * (double)nw.y;
-        G = make_double2(-by, bx);
-        if (q == q_mean) { F = make_double2(0.0, 0.0); G = F; }
-        if (g.fn > 0 && n == g.fn) {   // stochastic forcing of the step
-            const size_t o = ((size_t)mi * Ny + y) * E + e, half = (size_t)g.nkz * Ny * E;
-            F.x += g.noise[o].x; F.y += g.noise[o].y;
-            G.x += g.noise[half + o].x; G.y += g.noise[half + o].y;
-        }
-        size_t h = ((size_t)q * Ny + y) * E + e;
-        double2 Ft, Gt;
-        if (s == 0) {
-            Ft = F; Gt = G;
-            g.Av[h] = F; g.Ae[h] = G;
-        } else if (s == 1) {
-            double2 a = g.Av[h], b = g.Ae[h];
-            Ft = make_double2(2.0 * F.x - a.x, 2.0 * F.y - a.y);
-            Gt = make_double2(2.0 * G.x - b.x, 2.0 * G.y - b.y);
-            g.Av[h] = make_double2((1.0 / 6.0) * a.x + (4.0 / 6.0) * F.x, (1.0 / 6.0) * a.y + (4.0 / 6.0) * F.y);
-            g.Ae[h] = make_double2((1.0 / 6.0) * b.x + (4.0 / 6.0) * G.x, (1.0 / 6.0) * b.y + (4.0 / 6.0) * G.y);
-        } else {
-            double2 a = g.Av[h], b = g.Ae[h];
-            Ft = make_double2(a.x + (1.0 / 6.0) * F.x, a.y + (1.0 / 6.0) * F.y);
-            Gt = make_double2(b.x + (1.0 / 6.0) * G.x, b.y + (1.0 / 6.0) * G.y);
-        }
-        g.Fv[h] = Ft;
-        g.Fe[h] = Gt;
-    }
-}
-
-template <typename T>
-void launch_forcing(const GroupView& g, int s, cudaStream_t st) {
-    dim3 grid((g.nmodes + QB - 1) / QB, (g.E + EB - 1) / EB);
-    size_t smem = (size_t)QB * g.ny * EB * sizeof(typename C2<T>::type);
-    k_forcing<T><<<grid, 256, smem, st>>>(g, s);
-}
-template void launch_forcing<double>(const GroupView&, int, cudaStream_t);
 
 // --------------------------------------------------------------------- mean
 
@@ -208,89 +28,6 @@ __global__ void __launch_bounds__(128) k_mean_finish(GroupView g, int s) {
 void launch_mean_finish(const GroupView& g, int s, cudaStream_t st) {
     k_mean_finish<<<g.E, 128, 0, st>>>(g, s);
 }
-
-// --------------------------------------------------------------------- helm
-
-// stage: the pair's two operators are copied to shared memory (they fit up to
-// Ny = 120); above that every CTA reads them from global memory, where the
-// 2 npairs x 2 operators stay L2-resident across the CTAs of the launch.
-__global__ void __launch_bounds__(256) k_helm(GroupView g, int s, bool stage) {
-    extern __shared__ __align__(16) unsigned char sm[];
-    const int Ny = g.ny, E = g.E, NKX = g.nkx;
-    // leading CTAs: rows of the mean-flow update
-    const int nrow = mean_row_ctas(g);
-    if ((int)blockIdx.x < nrow) {
-        mean_rows(g, s, blockIdx.x % E, (blockIdx.x / E) * (blockDim.x >> 5), sm);
-        return;
-    }
-    const int b = blockIdx.x - nrow;
-    const int p = b % g.npairs, f = (b / g.npairs) & 1, ch = b / (2 * g.npairs);
-    const int n = p % NKX, am = p / NKX;
-    if (!g.lin && n == 0 && am == 0) return;   // the mean mode (DNS groups)
-    // members e0 .. e0 + ec - 1 (all of them unless the group is split into chunks)
-    const int EC = helm_member_chunk(g), e0 = ch * EC, ec = min(EC, E - e0);
-    const int hi = (s == 0) ? 0 : 1;
-    const size_t nn = (size_t)Ny * Ny;
-    const double* Mg = g.ops[hi] + ((size_t)p * 4 + (f == 0 ? 0 : 2)) * nn;
-    const double* Pg = Mg + nn;
-    const bool needM = (s != 2);
-    const double* Ms = Mg;
-    const double* Ps = Pg;
-    if (stage) {
-        double* ms = (double*)sm;
-        double* ps = ms + nn;
-        for (size_t i = threadIdx.x; i < nn; i += blockDim.x) {
-            if (needM) ms[i] = Mg[i];
-            ps[i] = Pg[i];
-        }
-        __syncthreads();
-        Ms = ms;
-        Ps = ps;
-    }
-    const int nq = am > 0 ? 2 : 1;
-    const int q1 = (g.kz + am) * NKX + n, q2 = (g.kz - am) * NKX + n;
-    const double2* X = f == 0 ? g.v_t : g.e_t;
-    const double2* F = f == 0 ? g.Fv : g.Fe;
-    double2* M1 = f == 0 ? g.mx1_v : g.mx1_e;
-    double2* O = (s == 2) ? (f == 0 ? g.v_t : g.e_t) : (f == 0 ? g.v_s : g.e_s);
-    const int ncol = 2 * E;                // real columns of a row in global memory
-    const int per = Ny * 2 * ec;
-    for (int idx = threadIdx.x; idx < nq * per; idx += blockDim.x) {
-        int which = idx / per;
-        int r = idx - which * per;
-        int y = r / (2 * ec), c = 2 * e0 + r - y * (2 * ec);
-        int q = which == 0 ? q1 : q2;
-        const double* xc = (const double*)(X + (size_t)q * Ny * E);
-        const double* fc = (const double*)(F + (size_t)q * Ny * E);
-        double* m1 = (double*)(M1 + (size_t)q * Ny * E);
-        double* oc = (double*)(O + (size_t)q * Ny * E);
-        double accP = 0.0;
-        const double* pr = Ps + (size_t)y * Ny;
-        for (int k = 0; k < Ny; ++k) accP += pr[k] * fc[k * ncol + c];
-        double out;
-        if (needM) {
-            double accM = 0.0;
-            const double* mr = Ms + (size_t)y * Ny;
-            for (int k = 0; k < Ny; ++k) accM += mr[k] * xc[k * ncol + c];
-            if (s == 1) m1[y * ncol + c] = accM;
-            out = accM + accP;
-        } else {
-            out = m1[y * ncol + c] + accP;
-        }
-        oc[y * ncol + c] = out;
-    }
-}
-
-void launch_helm(const GroupView& g, int s, cudaStream_t st) {
-    size_t smem = 2 * (size_t)g.ny * g.ny * sizeof(double);
-    const bool stage = smem <= 227 * 1024;
-    if (!stage) smem = 0;
-    if (smem < mean_smem_bytes(g)) smem = mean_smem_bytes(g);
-    k_helm<<<mean_row_ctas(g) + 2 * g.npairs * helm_member_chunks(g), 256, smem, st>>>(g, s, stage);
-}
-
-
-// --------------------------------------------------------------------- mean
 
 // -------------------------------------------------------------------- stats
 
@@ -522,14 +259,14 @@ void launch_shared_mean(const GroupView& g, bool fp64, cudaStream_t st) {
 }
 
 void launch_stats(const GroupView& g, cudaStream_t st) {
-    launch_yderiv<double>(g, g.v_t, g.e_t, g.P5d, st);
+    launch_yderiv64(g, g.v_t, g.e_t, g.P5d, st);
     k_stats_plane<<<dim3(g.ny, g.E), 256, 0, st>>>(g, g.st_y);
     if (!g.lin) k_stats_cfl<<<dim3(g.ny, g.E), 256, stats_cfl_smem_bytes(g), st>>>(g);
     k_stats_final<<<g.E, 128, 0, st>>>(g, g.st_y, g.st_out, 9, 1);
 }
 
 void launch_stats_packed(const GroupView& g, double* part, double* out, cudaStream_t st) {
-    launch_yderiv<double>(g, g.v_t, g.e_t, g.P5d, st);
+    launch_yderiv64(g, g.v_t, g.e_t, g.P5d, st);
     k_stats_plane<<<dim3(g.ny, g.E), 256, 0, st>>>(g, part);
     k_stats_final<<<g.E, 128, 0, st>>>(g, part, out, 8, 0);
 }
@@ -636,15 +373,12 @@ cudaError_t load_stats_kernels() {
     cudaFuncAttributes a;
     cudaError_t e = cudaFuncGetAttributes(&a, (const void*)k_stats_plane);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, (const void*)k_stats_final);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, (const void*)k_yderiv<double>);
+    if (e == cudaSuccess) e = load_yderiv64();
     return e;
 }
 
 void set_attributes_spectral() {
     allow_max_dynamic_smem(k_stats_cfl);
-    allow_max_dynamic_smem(k_yderiv<double>);
-    allow_max_dynamic_smem(k_forcing<double>);
-    allow_max_dynamic_smem(k_helm);
 }
 
 }  // namespace dnsk
