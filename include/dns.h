@@ -152,7 +152,7 @@ typedef struct {
                                       per plane with each 1-D transform owned by one group of
                                       threads (mixed precision, sizes <= 64), 5 three launches
                                       (z, x, z) that hand the planes on through L2 (both
-                                      precisions, sizes >= 32); a request for a variant the
+                                      precisions); a request for a variant the
                                       group's size lacks is ignored */
     int helm;                      /* mixed path per-wavenumber stage: 0 autotuned at
                                       dns_bind_workspace (DNS groups: 1, 2 and 8, each timed with

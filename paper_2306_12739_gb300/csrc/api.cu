@@ -533,8 +533,7 @@ bool plane_variant_ok(bool mixed, const GroupView& v, int c) {
 // kernel is asked for:
 //   128-point grids, where a plane does not fit one SM: 404 -> 153 us a launch
 //   against the cluster kernel on 128x97x128 x 4, 1099 -> 670 us in FP64;
-//   FP64 everywhere it can (grids of 32 points up): 991 -> 548 us on 64x65x64 x
-//   4, 154 -> 144 on 32x33x32 x 2; the single-CTA kernel spends its FP64 pipe on
+//   FP64 everywhere: 991 -> 548 us on 64x65x64 x 4, 154 -> 144 on 32x33x32 x 2; the single-CTA kernel spends its FP64 pipe on
 //   radix-2 to 4 passes and leaves SMs idle at few planes.
 bool plane_split_default(const GroupView& v, bool mixed) { return !mixed || v.mx == 128 || v.mz == 128; }
 
@@ -2150,8 +2149,17 @@ int dns_optimal_sweep(dns_handle* h, int nsteps, double* gains) {
     if ((rc = dns_step(h, nsteps))) return rc;
     launches += h->launches;
     if ((rc = dns_set_direction(h, -1, 0))) return rc;
-    for (auto& G : h->groups) {
-        launches += dnsk::launch_lin_orthonormalize(G.v, h->stream);
+    // the groups side by side: each on its own stream, as in a step
+    const bool multi = h->groups.size() > 1 && !h->gstreams.empty();
+    if (multi) cudaEventRecord(h->fork_ev, h->stream);
+    for (size_t gi = 0; gi < h->groups.size(); ++gi) {
+        cudaStream_t st = multi ? h->gstreams[gi] : h->stream;
+        if (multi) cudaStreamWaitEvent(st, h->fork_ev, 0);
+        launches += dnsk::launch_lin_orthonormalize(h->groups[gi].v, st);
+        if (multi) {
+            cudaEventRecord(h->gevents[gi], st);
+            cudaStreamWaitEvent(h->stream, h->gevents[gi], 0);
+        }
         if ((rc = check(h, cudaGetLastError(), "orthonormalize launch"))) return rc;
     }
     h->launches = launches;

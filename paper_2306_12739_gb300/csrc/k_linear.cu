@@ -21,10 +21,14 @@
 //   * modified Gram-Schmidt of the member set in the energy inner product
 //     <a, b> = (1/4) sum_q sum_j w_j (conj(v_a) v_b + (conj(Dv_a) Dv_b +
 //     conj(eta_a) eta_b) / k^2) over the interior nodes (w_j Clenshaw-Curtis
-//     weights, Dv = D1 v with v = 0 at the walls): one launch per vector k
-//     projects x_k out of every later vector (one CTA each) and normalises
-//     x_{k-1}, whose projections the previous launch completed.
+//     weights, Dv = D1 v with v = 0 at the walls), on contiguous copies of the
+//     vectors: one launch per vector k projects x_k out of every later vector, a
+//     thread-block cluster each.
 #include "dns_internal.hpp"
+#include "eo.cuh"
+#include <cooperative_groups.h>
+
+namespace cg = cooperative_groups;
 
 namespace dnsk {
 
@@ -183,106 +187,185 @@ void launch_lin_plane(const GroupView& g, bool fp64, cudaStream_t st) {
 
 // ------------------------------------------------------------ Gram-Schmidt
 
-// Dv = D1_int v for every member and kz (H layout, into the v_s scratch field)
-__global__ void __launch_bounds__(GS_THREADS) k_lin_dv(GroupView g) {
+// Why this form: a vector's elements lie E apart in the state, so one CTA per
+// vector reading them there drew half of every sector for nothing and left the
+// whole FP64 work of a vector (the pipe takes an SM about 16 cycles per warp
+// instruction) to one SM.  The vectors are gathered once, contiguous and scaled
+// to energy coordinates (sqrt of the weights), and a cluster of GS_CL CTAs
+// shares each projection: 45 vectors of 61 x 43 modes, per group 2.5 -> 0.25 ms.
+
+constexpr int GS_CL = 8;     // CTAs per vector
+constexpr int GS_EC = 8;     // members of a gather CTA
+
+// The three parts of a vector in energy coordinates, each [member][q Ny + y]:
+// v sqrt(w), Dv sqrt(w) / k, eta sqrt(w) / k.  They lie in arrays that a step
+// writes before it reads them (the sub-step states and a combined forcing).
+struct GsParts {
+    double2* y[3];
+};
+__host__ __device__ inline GsParts gs_parts(const GroupView& g) { return {{g.v_s, g.e_s, g.Fv}}; }
+
+__global__ void __launch_bounds__(GS_THREADS) k_gs_gather(GroupView g) {
     extern __shared__ __align__(16) unsigned char sm[];
-    double* D = (double*)sm;
-    const int Ny = g.ny, E = g.E, q = blockIdx.x;
-    for (int i = threadIdx.x; i < Ny * Ny; i += blockDim.x) D[i] = g.D1i[i];
-    __syncthreads();
-    const double2* v = g.v_t + (size_t)q * Ny * E;
-    double2* o = g.v_s + (size_t)q * Ny * E;
-    for (int i = threadIdx.x; i < Ny * E; i += blockDim.x) {
-        const int y = i / E, e = i - y * E;
-        double ax = 0.0, ay = 0.0;
-        for (int k = 0; k < Ny; ++k) {
-            const double d = D[y * Ny + k];
-            const double2 x = v[(size_t)k * E + e];
-            ax += d * x.x;
-            ay += d * x.y;
+    double2* X = (double2*)sm;                       // parity parts of v, then natural rows of v, eta [Ny][ec]
+    const int Ny = g.ny, E = g.E, q = blockIdx.x, e0 = blockIdx.y * GS_EC, ec = min(GS_EC, E - e0);
+    const int NE = (Ny + 1) / 2, NO = Ny / 2, RP = spc::eo_rp(Ny);
+    double2* VN = X + Ny * ec;
+    double2* HN = VN + Ny * ec;
+    for (int i = threadIdx.x; i < NE * ec; i += blockDim.x) {
+        const int p = i / ec, el = i - p * ec;
+        const spc::EoRows R = spc::eo_rows(p, Ny);
+        const size_t h0 = ((size_t)q * Ny + R.y0) * E + e0 + el, h1 = ((size_t)q * Ny + R.y1) * E + e0 + el;
+        const double2 a = g.v_t[h0];
+        VN[R.y0 * ec + el] = a;
+        HN[R.y0 * ec + el] = g.e_t[h0];
+        X[p * ec + el] = a;
+        if (R.pair) {
+            const double2 b = g.v_t[h1];
+            VN[R.y1 * ec + el] = b;
+            HN[R.y1 * ec + el] = g.e_t[h1];
+            X[p * ec + el] = make_double2(a.x + b.x, a.y + b.y);
+            X[(NE + p) * ec + el] = make_double2(a.x - b.x, a.y - b.y);
         }
-        o[i] = make_double2(ax, ay);
+    }
+    __syncthreads();
+    const double* D1e = g.D1EO64;                    // even output rows (contract the odd part), then the odd ones
+    const double* D1o = D1e + (size_t)NO * RP;
+    const GsParts Y = gs_parts(g);
+    const size_t n = (size_t)g.nmodes * Ny;
+    const double ik = sqrt(g.k2inv[q]);
+    for (int i = threadIdx.x; i < NE * ec; i += blockDim.x) {
+        const int el = i / NE, p = i - el * NE;      // consecutive threads: consecutive rows of a vector
+        double2 de = make_double2(0.0, 0.0), dd = de;
+#pragma unroll 4
+        for (int k = 0; k < NO; ++k) {
+            const double b = D1e[k * RP + p];
+            const double2 x = X[(NE + k) * ec + el];
+            de.x += b * x.x;
+            de.y += b * x.y;
+        }
+#pragma unroll 4
+        for (int k = 0; k < NE; ++k) {
+            const double b = D1o[k * RP + p];
+            const double2 x = X[k * ec + el];
+            dd.x += b * x.x;
+            dd.y += b * x.y;
+        }
+        const spc::EoRows R = spc::eo_rows(p, Ny);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            if (r && !R.pair) break;
+            const int y = r ? R.y1 : R.y0;
+            const double w = sqrt(g.ccw[y + 1]), wk = w * ik, h = R.pair ? 0.5 : 1.0, sg = !R.pair ? 0.0 : r ? -1.0 : 1.0;
+            const size_t o = (size_t)(e0 + el) * n + (size_t)q * Ny + y;
+            const double2 v = VN[y * ec + el], t = HN[y * ec + el];
+            Y.y[0][o] = make_double2(v.x * w, v.y * w);
+            Y.y[1][o] = make_double2(h * (de.x + sg * dd.x) * wk, h * (de.y + sg * dd.y) * wk);
+            Y.y[2][o] = make_double2(t.x * wk, t.y * wk);
+        }
     }
 }
 
-// launch k = 0 .. E: CTAs 0 .. E-k-2 take x_{k+1+b} -= (<x_k, x_j> / <x_k, x_k>) x_k
-// (v, eta and Dv); for k >= 1 the last CTA normalises x_{k-1} and records its
-// norm (energy, the 1/4 included).
-__global__ void __launch_bounds__(GS_THREADS) k_lin_gs(GroupView g, int k) {
+// Sum of a CTA value over its cluster, in rank order, in every CTA.  part: two
+// doubles of this CTA's shared memory.
+__device__ __forceinline__ double2 cluster_sum(double2 v, double2* part, double* red) {
+    cg::cluster_group cl = cg::this_cluster();
+    v.x = block_sum(v.x, red);
+    v.y = block_sum(v.y, red);
+    if (threadIdx.x == 0) *part = v;
+    cl.sync();
+    double2 s = make_double2(0.0, 0.0);
+    for (int r = 0; r < GS_CL; ++r) {
+        const double2 t = *cl.map_shared_rank(part, r);
+        s.x += t.x;
+        s.y += t.y;
+    }
+    return s;
+}
+
+// Launch k = -1: the squared norm of x_0.  Launch k >= 0: cluster b takes
+// x_j -= (<x_k, x_j> / <x_k, x_k>) x_k for j = k + 1 + b; x_{k+1} then has all its
+// projections, and its squared norm is recorded.
+__global__ void __cluster_dims__(GS_CL, 1, 1) __launch_bounds__(GS_THREADS) k_gs_project(GroupView g, int k) {
     __shared__ double red[32];
-    const int E = g.E, Ny = g.ny, NM = g.nmodes;
-    const int nproj = k < E ? E - k - 1 : 0;
-    const double* w = g.ccw + 1;
-    double2* V = g.v_t;
-    double2* H = g.e_t;
-    double2* DV = g.v_s;
-    const int n = NM * Ny;   // elements of one vector per field, H index (q Ny + y) E + member
-    if ((int)blockIdx.x < nproj) {
-        const int j = k + 1 + blockIdx.x;
-        double nn = 0.0, cr = 0.0, ci = 0.0;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const int q = i / Ny, y = i - q * Ny;
-            const double wy = w[y], wk = wy * g.k2inv[q];
-            const size_t hk = (size_t)i * E + k, hj = (size_t)i * E + j;
-            const double2 a0 = V[hk], b0 = V[hj], a1 = DV[hk], b1 = DV[hj], a2 = H[hk], b2 = H[hj];
-            nn += wy * (a0.x * a0.x + a0.y * a0.y) + wk * (a1.x * a1.x + a1.y * a1.y + a2.x * a2.x + a2.y * a2.y);
-            cr += wy * (a0.x * b0.x + a0.y * b0.y) + wk * (a1.x * b1.x + a1.y * b1.y + a2.x * b2.x + a2.y * b2.y);
-            ci += wy * (a0.x * b0.y - a0.y * b0.x) + wk * (a1.x * b1.y - a1.y * b1.x + a2.x * b2.y - a2.y * b2.x);
-        }
-        nn = block_sum(nn, red);
-        cr = block_sum(cr, red);
-        ci = block_sum(ci, red);
-        const double cx = cr / nn, cy = ci / nn;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const size_t hk = (size_t)i * E + k, hj = (size_t)i * E + j;
-            double2* arr[3] = {V, DV, H};
+    __shared__ double2 part[2];
+    const int j = k + 1 + blockIdx.x / GS_CL;
+    const GsParts Y = gs_parts(g);
+    const size_t n = (size_t)g.nmodes * g.ny;
+    const int step = GS_CL * GS_THREADS, i0 = (int)cg::this_cluster().block_rank() * GS_THREADS + threadIdx.x;
+    double2 c = make_double2(0.0, 0.0);
+    if (k >= 0) {
+        double2 s = make_double2(0.0, 0.0);
 #pragma unroll
-            for (int f = 0; f < 3; ++f) {
-                const double2 a = arr[f][hk];
-                double2 b = arr[f][hj];
-                b.x -= cx * a.x - cy * a.y;
-                b.y -= cx * a.y + cy * a.x;
-                arr[f][hj] = b;
+        for (int f = 0; f < 3; ++f) {
+            const double2 *xk = Y.y[f] + (size_t)k * n, *xj = Y.y[f] + (size_t)j * n;
+#pragma unroll 2
+            for (int i = i0; i < (int)n; i += step) {
+                const double2 a = xk[i], b = xj[i];
+                s.x += a.x * b.x + a.y * b.y;
+                s.y += a.x * b.y - a.y * b.x;
             }
         }
-    } else {
-        const int j = k - 1;
-        double nn = 0.0;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const int q = i / Ny, y = i - q * Ny;
-            const double wy = w[y], wk = wy * g.k2inv[q];
-            const size_t hj = (size_t)i * E + j;
-            const double2 a0 = V[hj], a1 = DV[hj], a2 = H[hj];
-            nn += wy * (a0.x * a0.x + a0.y * a0.y) + wk * (a1.x * a1.x + a1.y * a1.y + a2.x * a2.x + a2.y * a2.y);
-        }
-        nn = block_sum(nn, red);
-        const double r = sqrt(0.25 * nn);
-        if (threadIdx.x == 0) g.gsr[j] = r;
-        const double s = 1.0 / r;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const size_t hj = (size_t)i * E + j;
-            V[hj] = make_double2(V[hj].x * s, V[hj].y * s);
-            H[hj] = make_double2(H[hj].x * s, H[hj].y * s);
+        s = cluster_sum(s, part, red);
+        const double nn = g.gsr[k];
+        c = make_double2(s.x / nn, s.y / nn);
+    }
+    const bool norm = j == k + 1;
+    double2 s = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+        const double2* xk = Y.y[f] + (size_t)(k < 0 ? 0 : k) * n;
+        double2* xj = Y.y[f] + (size_t)j * n;
+#pragma unroll 2
+        for (int i = i0; i < (int)n; i += step) {
+            double2 b = xj[i];
+            if (k >= 0) {
+                const double2 a = xk[i];
+                b.x -= c.x * a.x - c.y * a.y;
+                b.y -= c.x * a.y + c.y * a.x;
+                xj[i] = b;
+            }
+            if (norm) s.x += b.x * b.x + b.y * b.y;
         }
     }
+    if (norm) {
+        s = cluster_sum(s, part + 1, red);
+        if (cg::this_cluster().block_rank() == 0 && threadIdx.x == 0) g.gsr[j] = s.x;
+    }
+    cg::this_cluster().sync();       // no CTA leaves while a peer may still read its part
+}
+
+// Every vector normalised and back in the state; its energy norm (the 1/4
+// included) recorded after the last CTA has read the squared norms.
+__global__ void __launch_bounds__(GS_THREADS) k_gs_scatter(GroupView g) {
+    const int Ny = g.ny, E = g.E, q = blockIdx.x;
+    const GsParts Y = gs_parts(g);
+    const size_t n = (size_t)g.nmodes * Ny;
+    const double k1 = sqrt(1.0 / g.k2inv[q]);
+    for (int i = threadIdx.x; i < Ny * E; i += blockDim.x) {
+        const int y = i / E, e = i - y * E;
+        const double s = 1.0 / (sqrt(0.25 * g.gsr[e]) * sqrt(g.ccw[y + 1]));
+        const size_t o = (size_t)e * n + (size_t)q * Ny + y, h = ((size_t)q * Ny + y) * E + e;
+        const double2 a = Y.y[0][o], b = Y.y[2][o];
+        g.v_t[h] = make_double2(a.x * s, a.y * s);
+        g.e_t[h] = make_double2(b.x * (s * k1), b.y * (s * k1));
+    }
+}
+__global__ void k_gs_norms(GroupView g) {
+    for (int e = threadIdx.x; e < g.E; e += blockDim.x) g.gsr[e] = sqrt(0.25 * g.gsr[e]);
 }
 
 int launch_lin_orthonormalize(const GroupView& g, cudaStream_t st) {
-    k_lin_dv<<<g.nmodes, GS_THREADS, sizeof(double) * (size_t)g.ny * g.ny, st>>>(g);
-    int launches = 1;
-    for (int k = 0; k <= g.E; ++k) {
-        const int nproj = k < g.E ? g.E - k - 1 : 0;
-        const int grid = nproj + (k >= 1 ? 1 : 0);
-        if (grid > 0) {
-            k_lin_gs<<<grid, GS_THREADS, 0, st>>>(g, k);
-            ++launches;
-        }
-    }
-    return launches;
+    const size_t smem = 3 * (size_t)g.ny * GS_EC * sizeof(double2);
+    k_gs_gather<<<dim3(g.nmodes, (g.E + GS_EC - 1) / GS_EC), GS_THREADS, smem, st>>>(g);
+    for (int k = -1; k < g.E - 1; ++k) k_gs_project<<<GS_CL * (k < 0 ? 1 : g.E - 1 - k), GS_THREADS, 0, st>>>(g, k);
+    k_gs_scatter<<<g.nmodes, GS_THREADS, 0, st>>>(g);
+    k_gs_norms<<<1, 64, 0, st>>>(g);
+    return g.E + 3;
 }
 
 void set_attributes_linear() {
-    allow_max_dynamic_smem(k_lin_dv);
+    allow_max_dynamic_smem(k_gs_gather);
     // the plane stage needs at most 2 x 9 x 128 x 16 B = 36 KB, below the default limit
 }
 

@@ -74,6 +74,8 @@ constexpr int ZTHREADS = 128;                                 // most threads of
 // columns of a CTA: the tiles of a plane as equal as they come within ZTHREADS
 __host__ __device__ constexpr int ztiles(int nkx, int h) { return (nkx * h + ZTHREADS - 1) / ZTHREADS; }
 __host__ __device__ constexpr int ztile(int nkx, int h) { return (nkx + ztiles(nkx, h) - 1) / ztiles(nkx, h); }
+// threads of a CTA: at least one whole warp (rows j >= H idle)
+__host__ __device__ constexpr int zthreads(int tn, int h) { return tn * h < 32 ? 32 : tn * h; }
 // stride of the k1 rows of the exchange, = TN modulo 8: two neighbouring rows
 // then fall in the 16-byte banks as if contiguous
 template <int MZ>
@@ -116,7 +118,7 @@ k_ps_zinv(GroupView g, const double* __restrict__ Ucur, const double* __restrict
     const int tid = threadIdx.x, j = tid / TN, nl = tid - j * TN;
     const int pe = blockIdx.x, y = pe / g.E, e = pe - y * g.E, n = blockIdx.y * TN + nl;
     const size_t fs = (size_t)g.ny * g.E * g.nmodes;
-    const bool act = n < nkx;
+    const bool row = j < H, act = row && n < nkx;
     if (!DNS_CK(g.status, y < g.ny && MZ == g.mz, CK_PLANE_SPLIT, pe)) return;
     const C* __restrict__ P = (const C*)g.P5 + (size_t)pe * g.nmodes + (act ? n : 0);
     Pc<T>* __restrict__ col = (Pc<T>*)g.COL + (size_t)pe * NF * HP * NS + n;
@@ -203,14 +205,17 @@ k_ps_zinv(GroupView g, const double* __restrict__ Ucur, const double* __restrict
             }
             Pc<T>* Xb = X + (c & 1) * N1 * KS;
             Pc<T>* x = Xb + j * TN + nl;
-            pdft_padded<N1, +1>(v);
+            if (row) {
+                pdft_padded<N1, +1>(v);
 #pragma unroll
-            for (int k1 = 0; k1 < N1; ++k1) stp(x + k1 * KS, k1 == 0 ? v[0] : pmul<true>(v[k1], ldp(tw + k1 * H + j)));
+                for (int k1 = 0; k1 < N1; ++k1)
+                    stp(x + k1 * KS, k1 == 0 ? v[0] : pmul<true>(v[k1], ldp(tw + k1 * H + j)));
+            }
             __syncthreads();
 #pragma unroll
             for (int q = 0; q < K::NQ; ++q) {
                 const int k1 = j + H * q;
-                if (K::NQ * H > N1 && k1 >= N1) continue;
+                if (!row || (K::NQ * H > N1 && k1 >= N1)) continue;
                 const Pc<T>* xr = Xb + k1 * KS + nl;
                 Pc<T> o[H];
 #pragma unroll
@@ -241,7 +246,7 @@ k_ps_zfwd(GroupView g, int parts) {
     Pc<T>* X = tw + N1 * H;
     const int tid = threadIdx.x, j = tid / TN, nl = tid - j * TN;
     const int pe = blockIdx.x, n = blockIdx.y * TN + nl, f = blockIdx.z;
-    const bool act = n < nkx;
+    const bool row = j < H, act = row && n < nkx;
     if (!DNS_CK(g.status, pe < g.ny * g.E && MZ == g.mz, CK_PLANE_SPLIT, pe)) return;
     if (f == 0 && blockIdx.y == 0 && tid == 0) {
         // plane means <uv>, <wv>: the line pairs' partial sums in a fixed order
@@ -260,7 +265,7 @@ k_ps_zfwd(GroupView g, int parts) {
 #pragma unroll
     for (int q = 0; q < K::NQ; ++q) {
         const int k1 = j + H * q;
-        if (K::NQ * H > N1 && k1 >= N1) continue;
+        if (!row || (K::NQ * H > N1 && k1 >= N1)) continue;
 #pragma unroll
         for (int k = 0; k < H; ++k) v[q][k] = ldp(col + (size_t)(k1 + N1 * k) * NS);
     }
@@ -268,7 +273,7 @@ k_ps_zfwd(GroupView g, int parts) {
 #pragma unroll
     for (int q = 0; q < K::NQ; ++q) {
         const int k1 = j + H * q;
-        if (K::NQ * H > N1 && k1 >= N1) continue;
+        if (!row || (K::NQ * H > N1 && k1 >= N1)) continue;
         dft_dif<N2, -1>(v[q]);
         Pc<T>* x = X + k1 * KS + nl;
 #pragma unroll
@@ -309,6 +314,7 @@ template <int MX> struct XCfg {
     static constexpr int R0 = N1 * XS > H * XF ? N1 * XS : H * XF;
     static constexpr int RS = H == 4 ? R0 + ((4 - R0 % 8) + 8) % 8 : R0;
     static constexpr int PH = NQ * H;                         // point pairs per lane
+    static constexpr bool RAGGED = H == 2;                    // a warp may hold more line pairs than a plane has
     static_assert(2 * NL <= N1, "kept coefficients and their mirrors fill distinct slots");
 };
 constexpr int XWARPS = 4;   // most warps of a CTA
@@ -336,7 +342,8 @@ k_ps_x(GroupView g) {
     Pc<T>* X = tw + N1 * XS + warp * xwarp_pairs<MX>(ROT) + (ROT ? 5 : 3) * PH * 32 + (lane / H) * K::RS;
     const int pe = blockIdx.x, HP = g.mz / 2, NS = col_row(K::KX + 1);
     const int p = (blockIdx.y * (blockDim.x >> 5) + warp) * K::L + lane / H;
-    if (!DNS_CK(g.status, pe < g.ny * g.E && p < HP && MX == g.mx, CK_PLANE_SPLIT, pe)) return;
+    const bool act = !K::RAGGED || p < HP;
+    if (!DNS_CK(g.status, pe < g.ny * g.E && (p < HP || K::RAGGED) && MX == g.mx, CK_PLANE_SPLIT, pe)) return;
     for (int i = tid; i < N1 * H; i += blockDim.x) {
         const int k1 = i / H, j = i - k1 * H;
         const auto a = Tab<T>::twx(g)[j * k1], b = Tab<T>::twx(g)[(j ? N2 - j : H) * k1];
@@ -369,8 +376,8 @@ k_ps_x(GroupView g) {
         for (int j = 0; j < NL; ++j) {
             const int ka = N2 * j + t, kb = N2 * j + nb;
             A[j] = B[j] = {dup((T)0), dup((T)0)};
-            if (ka <= KX) A[j] = ldp(r + ka);
-            if (kb <= KX) B[j] = ldp(r + kb);
+            if (act && ka <= KX) A[j] = ldp(r + ka);
+            if (act && kb <= KX) B[j] = ldp(r + kb);
         }
     };
     // the loaded line pair (times i kx for dx) inverse transformed: o[q H + m] holds
@@ -456,9 +463,9 @@ k_ps_x(GroupView g) {
             const int ka = N2 * j + t, kb = N2 * j + nb;
             const Pc<T> u = v[N1 - 1 - j], s = v[(N1 - j) % N1];
             const T wx = v[j].x.a, wy = v[j].y.a, cx = t ? u.x.b : s.x.a, cy = t ? u.y.b : s.y.a;
-            if (ka <= KX) stp(r + ka, Pc<T>{pr((wx + cx) * sx, (wy + cy) * sx), pr((wy - cy) * sx, (cx - wx) * sx)});
+            if (act && ka <= KX) stp(r + ka, Pc<T>{pr((wx + cx) * sx, (wy + cy) * sx), pr((wy - cy) * sx, (cx - wx) * sx)});
             const T zx = v[j].x.b, zy = v[j].y.b, dx = t ? u.x.a : u.x.b, dy = t ? u.y.a : u.y.b;
-            if (kb <= KX) stp(r + kb, Pc<T>{pr((zx + dx) * sx, (zy + dy) * sx), pr((zy - dy) * sx, (dx - zx) * sx)});
+            if (act && kb <= KX) stp(r + kb, Pc<T>{pr((zx + dx) * sx, (zy + dy) * sx), pr((zy - dy) * sx, (dx - zx) * sx)});
         }
         __syncwarp();
     };
@@ -555,19 +562,22 @@ k_ps_x(GroupView g) {
     if (tid == 0) g.psum[(size_t)pe * gridDim.y + blockIdx.y] = make_double2(suv, swv);
 }
 
-// warps of a k_ps_x CTA: the most, up to XWARPS, that divide the plane's line pairs
+// warps of a k_ps_x CTA: the most, up to XWARPS, that divide the plane's warps
+// (0: line pairs the lanes of a warp do not divide)
+template <int MX> constexpr int xplane_warps(int mz) {
+    return (mz / 2 + XCfg<MX>::L - 1) / XCfg<MX>::L;
+}
 template <int MX>
 int xwarps(int mz) {
-    const int hp = mz / 2, L = XCfg<MX>::L;
-    if (hp % L) return 0;
+    if (!XCfg<MX>::RAGGED && mz / 2 % XCfg<MX>::L) return 0;
     for (int w = XWARPS; w > 0; --w)
-        if (hp / L % w == 0) return w;
+        if (xplane_warps<MX>(mz) % w == 0) return w;
     return 0;
 }
 
 template <typename T, int MX, bool ROT>
 int launch_x(const GroupView& g, cudaStream_t st) {
-    const int w = xwarps<MX>(g.mz), parts = g.mz / 2 / XCfg<MX>::L / w;
+    const int w = xwarps<MX>(g.mz), parts = xplane_warps<MX>(g.mz) / w;
     k_ps_x<T, MX, ROT><<<dim3(g.ny * g.E, parts), 32 * w, xsmem<MX, T>(w, ROT), st>>>(g);
     return parts;
 }
@@ -576,19 +586,19 @@ template <typename T, int MZ>
 void launch_zinv(const GroupView& g, const double* U, const double* W, cudaStream_t st) {
     const int tn = ztile(g.nkx, ZCfg<MZ>::H);
     const dim3 grid(g.ny * g.E, (g.nkx + tn - 1) / tn, 3);
-    if (g.rot) k_ps_zinv<T, MZ, true><<<grid, ZCfg<MZ>::H * tn, zsmem<MZ, T>(g.nkx, 2), st>>>(g, U, W);
-    else k_ps_zinv<T, MZ, false><<<grid, ZCfg<MZ>::H * tn, zsmem<MZ, T>(g.nkx, 2), st>>>(g, U, W);
+    if (g.rot) k_ps_zinv<T, MZ, true><<<grid, zthreads(tn, ZCfg<MZ>::H), zsmem<MZ, T>(g.nkx, 2), st>>>(g, U, W);
+    else k_ps_zinv<T, MZ, false><<<grid, zthreads(tn, ZCfg<MZ>::H), zsmem<MZ, T>(g.nkx, 2), st>>>(g, U, W);
 }
 template <typename T, int MZ>
 void launch_zfwd(const GroupView& g, int parts, cudaStream_t st) {
     const int tn = ztile(g.nkx, ZCfg<MZ>::H);
     const dim3 grid(g.ny * g.E, (g.nkx + tn - 1) / tn, 3);
-    k_ps_zfwd<T, MZ><<<grid, ZCfg<MZ>::H * tn, zsmem<MZ, T>(g.nkx, 1), st>>>(g, parts);
+    k_ps_zfwd<T, MZ><<<grid, zthreads(tn, ZCfg<MZ>::H), zsmem<MZ, T>(g.nkx, 1), st>>>(g, parts);
 }
 
 }  // namespace psp
 
-#define DNS_SPLIT_LENGTHS(X) X(32) X(48) X(64) X(128)
+#define DNS_SPLIT_LENGTHS(X) X(16) X(32) X(48) X(64) X(128)
 
 bool plane_split_supported(const GroupView& g) {
     if (g.lin || (g.rot && (g.mx == 128 || g.mz == 128))) return false;

@@ -53,6 +53,13 @@ template <bool CONJ, typename T> __device__ __forceinline__ Pc<T> pmul(Pc<T> p, 
 // In-register DFTs of R points, natural order in and out, kernel
 // exp(S 2 pi i jk / R).  MID0: points 3 and 4 of 8 are zero (padding).
 template <int R, int S, typename T> struct Pdft;
+template <int S, typename T> struct Pdft<2, S, T> {
+    __device__ __forceinline__ static void run(Pc<T>* v) {
+        const Pc<T> a = v[0] + v[1];
+        v[1] = v[0] - v[1];
+        v[0] = a;
+    }
+};
 template <int S, typename T> struct Pdft<3, S, T> {
     __device__ __forceinline__ static void run(Pc<T>* v) {
         const Pr<T> h = dup((T)0.86602540378443864676), m = dup((T)-0.5);
@@ -118,7 +125,7 @@ template <int R, int S, typename T> __device__ __forceinline__ void pdft_padded(
     else Pdft<R, S, T>::run(v);
 }
 
-// (x, y) exp(S 2 pi i j / N), N = 8 or 16, j < N / 2 a compile-time value after unrolling
+// (x, y) exp(S 2 pi i j / N), N = 4, 8 or 16, j < N / 2 a compile-time value after unrolling
 template <int N, int S, typename T> __device__ __forceinline__ void rot_const(int j, T& x, T& y) {
     const T c1 = (T)0.92387953251128675613, s1 = (T)0.38268343236508977173, c2 = (T)0.70710678118654752440;
     const T cs[8] = {(T)1, c1, c2, s1, (T)0, -s1, -c2, -c1}, sn[8] = {(T)0, s1, c2, c1, (T)1, c1, c2, s1};
@@ -131,7 +138,7 @@ template <int N, int S, typename T> __device__ __forceinline__ void rot_const(in
     y = y0 * c + x0 * s;
 }
 
-// One N-point DFT (N = 8, 16) of a single transform, its halves as the two lanes.
+// One N-point DFT (N = 4, 8, 16) of a single transform, its halves as the two lanes.
 // Decimation in time: lanes (2 m, 2 m + 1) in, (k, k + N / 2) out.
 template <int N, int S, typename T> __device__ __forceinline__ void dft_dit(Pc<T>* v) {
     Pdft<N / 2, S, T>::run(v);

@@ -11,7 +11,8 @@ import oracle.dns as oracle
 pytestmark = pytest.mark.gpu
 dns = pytest.importorskip("paper_2306_12739_gb300")
 
-SIZES = [(32, 9, 32, 3, "advective"), (32, 6, 128, 1, "advective"), (48, 11, 32, 2, "rotational"),
+SIZES = [(16, 7, 16, 3, "advective"), (16, 6, 48, 1, "rotational"), (48, 7, 16, 2, "advective"),
+         (32, 9, 32, 3, "advective"), (32, 6, 128, 1, "advective"), (48, 11, 32, 2, "rotational"),
          (48, 5, 64, 1, "advective"), (64, 8, 48, 3, "advective"), (64, 9, 64, 2, "rotational"),
          (64, 6, 128, 2, "advective"), (128, 7, 64, 1, "advective"), (128, 9, 128, 2, "advective")]
 
