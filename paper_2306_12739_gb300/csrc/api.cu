@@ -160,7 +160,7 @@ bool eo_candidate(const GroupView& v) { return (v.helm == 4 || v.helm == 0) && e
 // the step-by-step forcing and apply in parity blocks may run (a request, helm
 // 8, or the autotuner): they read the pair operators and D1 in parity blocks
 bool step_eo_candidate(const GroupView& v) {
-    return (v.helm == 0 || (v.helm == 1 && v.step_eo)) && dnsk::step_eo_supported(v);
+    return (v.helm == 0 || (v.helm == 1 && v.step_eo)) && dnsk::step_eo_fits(v);
 }
 bool eo_images(const GroupView& v) { return eo_candidate(v) || step_eo_candidate(v); }
 
@@ -288,7 +288,7 @@ size_t layout_group(dns_handle* h, HostGroup& G, size_t cur) {
     }
     if (v.lin) {
         add((void**)&v.dir, 256);
-        add((void**)&v.gsr, sizeof(double) * v.E);
+        add((void**)&v.gsr, sizeof(double) * 3 * v.E);
         add((void**)&v.base, sizeof(double) * 9 * (size_t)v.ny * v.mz);
         if (precision_mixed(h)) add((void**)&v.basef, sizeof(float) * 9 * (size_t)v.ny * v.mz);
     }
@@ -1219,43 +1219,36 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
             if (v.helm == 4) v.ygemm = 1;
         }
     }
-    // linear groups: the apply kernels alone
+    // linear groups: the forcing and the apply, alone
     for (auto& G : h->groups) {
         GroupView& v = G.v;
         if (v.helm != 0) continue;
         const std::string key = tune_helm_key(v);
         int choice = decided.count(key) ? decided[key] : cache_lookup(h->cfg.autotune_cache, key);
-        if ((choice == 2 && !dnsk::helm_tc_supported(v)) || (choice == 4 && (v.lin || !dnsk::spec_supported(v))) || choice == 3)
+        const bool eo8 = step_eo_candidate(v) && v.opsEO[0] != nullptr && v.D1EO != nullptr;
+        if ((choice == 2 && !dnsk::helm_tc_supported(v)) || (choice == 8 && !eo8) || (choice > 2 && choice != 8))
             choice = 0;
         if (!choice) {
-            // the implicit apply is timed on sub-step 2 (both accumulators); it
-            // writes only the sub-step state, which set_state overwrites later
-            float best[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+            // timed on sub-step 2 (both accumulators); it writes only the sub-step
+            // state, which set_state overwrites later
+            float best[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             cudaEvent_t e0, e1;
             cudaEventCreate(&e0);
             cudaEventCreate(&e1);
-            // the persistent variant (3) fills the whole GPU, which timed alone
-            // wins but inside the step starves the concurrent member blocks and
-            // groups: only on request, never autotuned.  A DNS group times the
-            // whole per-wavenumber part of a sub-step: the y-derivatives, the
-            // forcing and the apply (1, 2) against the fused stage (4).
-            const bool whole = !v.lin;
-            for (int cand = 1; cand <= 4; ++cand) {
+            // the persistent variant (3) fills the whole GPU, which starves the
+            // concurrent groups: only on request.  8: forcing and apply in parity
+            // blocks (the implicit operators hold no base flow, so they have the
+            // reflection symmetry in a linear group too).
+            for (int cand : {1, 2, 8}) {
                 if (cand == 2 && !dnsk::helm_tc_supported(v)) continue;
-                if (cand == 3) continue;
-                if (cand == 4 && !(whole && dnsk::spec_supported(v))) continue;
+                if (cand == 8 && !eo8) continue;
                 auto run = [&]() {
-                    if (cand == 4) {
-                        dnsk::launch_spec(v, 1, st);
-                        if (v.d2tc && !v.d2fuse) dnsk::launch_d2v_tc(v, v.v_s, st);
+                    if (cand == 8) {
+                        dnsk::launch_forcing_eo(v, 1, st);
+                        dnsk::launch_helm_eo(v, 1, st);
                         return;
                     }
-                    if (whole) {
-                        if (v.ygemm == 2) dnsk::launch_yderiv_tc(v, v.v_t, v.e_t, st);
-                        else if (v.ygemm == 3) dnsk::launch_yderiv_eo(v, v.v_t, v.e_t, st);
-                        else dnsk::launch_yderiv_t(v, v.v_t, v.e_t, st);
-                        dnsk::launch_forcing_t(v, 1, st);
-                    }
+                    dnsk::launch_forcing_t(v, 1, st);
                     if (cand == 2) dnsk::launch_helm_tc(v, 1, st);
                     else dnsk::launch_helm_t(v, 1, st);
                 };
@@ -1273,13 +1266,13 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
             if (rc) return rc;
             if ((rc = device_status(h))) return rc;
             choice = 0;
-            for (int cand = 1; cand <= 4; ++cand)
+            for (int cand : {1, 2, 8})
                 if (best[cand] > 0.f && (choice == 0 || best[cand] < best[choice])) choice = cand;
-            cache_store(h->cfg.autotune_cache, key, choice, best, 4);
+            cache_store(h->cfg.autotune_cache, key, choice, best, 8);
         }
         decided[key] = choice;
-        v.helm = choice;
-        if (choice == 4) v.ygemm = 1;
+        v.helm = choice == 8 ? 1 : choice;
+        v.step_eo = choice == 8 ? 1 : 0;
     }
     // Tile shapes (neither changes a result: every column is computed the same
     // way whatever tile holds it).  Members per CTA of the fused stage:

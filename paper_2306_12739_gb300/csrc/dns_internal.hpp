@@ -38,7 +38,7 @@ struct GroupView {
     const double* base;   // linear groups: [9][Ny][Mz] U, V, W, d_y(U, V, W), d_z(U, V, W) of the
                           //    base flow on the interior planes
     const float* basef;   // single-precision copy (mixed path)
-    double* gsr;          // linear groups: [E] energy norms recorded by the last Gram-Schmidt
+    double* gsr;          // linear groups: [3][E], the first row the energy norms of the last Gram-Schmidt
     // stochastic forcing (DNS groups; fn = 0: off)
     int fn;               // forced streamwise index
     int fneig;            // structures per block (v, eta) and kz
@@ -196,6 +196,7 @@ void set_attributes_spec();
 bool yderiv_eo_supported(const GroupView& g);
 size_t yderiv_eo_smem_bytes(const GroupView& g);
 void launch_yderiv_eo(const GroupView& g, const double2* v, const double2* e, cudaStream_t st, int sprev = -1);
+bool step_eo_fits(const GroupView& g);
 bool step_eo_supported(const GroupView& g);
 size_t forcing_eo_smem_bytes(const GroupView& g);
 size_t helm_eo_smem_bytes(const GroupView& g);

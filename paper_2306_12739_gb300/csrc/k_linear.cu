@@ -196,6 +196,7 @@ void launch_lin_plane(const GroupView& g, bool fp64, cudaStream_t st) {
 
 constexpr int GS_CL = 8;     // CTAs per vector
 constexpr int GS_EC = 8;     // members of a gather CTA
+constexpr int GS_B = 4;      // elements of a thread in flight
 
 // The three parts of a vector in energy coordinates, each [member][q Ny + y]:
 // v sqrt(w), Dv sqrt(w) / k, eta sqrt(w) / k.  They lie in arrays that a step
@@ -204,6 +205,10 @@ struct GsParts {
     double2* y[3];
 };
 __host__ __device__ inline GsParts gs_parts(const GroupView& g) { return {{g.v_s, g.e_s, g.Fv}}; }
+// g.gsr: [3][E] norms, squared norms' reciprocals, squared norms
+__device__ __forceinline__ double* gs_norm(const GroupView& g) { return g.gsr; }
+__device__ __forceinline__ double* gs_inv(const GroupView& g) { return g.gsr + g.E; }
+__device__ __forceinline__ double* gs_sq(const GroupView& g) { return g.gsr + 2 * g.E; }
 
 __global__ void __launch_bounds__(GS_THREADS) k_gs_gather(GroupView g) {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -266,102 +271,156 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs_gather(GroupView g) {
     }
 }
 
-// Sum of a CTA value over its cluster, in rank order, in every CTA.  part: two
-// doubles of this CTA's shared memory.
-__device__ __forceinline__ double2 cluster_sum(double2 v, double2* part, double* red) {
+// Sum of the threads' values over the cluster, in a fixed order, times f; the
+// result in every thread.  On the FP64 pipe an addition costs a warp 16 cycles
+// of its SM, so one warp adds up the CTA and one thread the cluster.
+struct GsShared {
+    double2 lane[GS_THREADS];
+    double2 part, sum;
+};
+__device__ __forceinline__ double2 cluster_sum(double2 v, double f, GsShared& sh) {
     cg::cluster_group cl = cg::this_cluster();
-    v.x = block_sum(v.x, red);
-    v.y = block_sum(v.y, red);
-    if (threadIdx.x == 0) *part = v;
-    cl.sync();
-    double2 s = make_double2(0.0, 0.0);
-    for (int r = 0; r < GS_CL; ++r) {
-        const double2 t = *cl.map_shared_rank(part, r);
-        s.x += t.x;
-        s.y += t.y;
+    sh.lane[threadIdx.x] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        double2 t = sh.lane[threadIdx.x];
+#pragma unroll
+        for (int i = 32; i < GS_THREADS; i += 32) {
+            const double2 u = sh.lane[threadIdx.x + i];
+            t.x += u.x;
+            t.y += u.y;
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+            t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+        }
+        if (threadIdx.x == 0) sh.part = t;
     }
-    return s;
+    cl.sync();
+    if (threadIdx.x == 0) {
+        double2 t = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int r = 0; r < GS_CL; ++r) {
+            const double2 u = *cl.map_shared_rank(&sh.part, r);
+            t.x += u.x;
+            t.y += u.y;
+        }
+        sh.sum = make_double2(t.x * f, t.y * f);
+    }
+    cl.sync();       // the sum is there, and no peer reads this CTA's part any more
+    return sh.sum;
 }
 
 // Launch k = -1: the squared norm of x_0.  Launch k >= 0: cluster b takes
 // x_j -= (<x_k, x_j> / <x_k, x_k>) x_k for j = k + 1 + b; x_{k+1} then has all its
-// projections, and its squared norm is recorded.
-__global__ void __cluster_dims__(GS_CL, 1, 1) __launch_bounds__(GS_THREADS) k_gs_project(GroupView g, int k) {
-    __shared__ double red[32];
-    __shared__ double2 part[2];
-    const int j = k + 1 + blockIdx.x / GS_CL;
+// projections, and its squared norm and its reciprocal are recorded.
+__global__ void __cluster_dims__(GS_CL, 1, 1) __launch_bounds__(GS_THREADS, 3) k_gs_project(GroupView g, int k) {
+    __shared__ GsShared sh;
+    const int j = k + 1 + blockIdx.x / GS_CL, rank = blockIdx.x % GS_CL;
     const GsParts Y = gs_parts(g);
-    const size_t n = (size_t)g.nmodes * g.ny;
-    const int step = GS_CL * GS_THREADS, i0 = (int)cg::this_cluster().block_rank() * GS_THREADS + threadIdx.x;
+    const int n = g.nmodes * g.ny, n3 = 3 * n, step = GS_CL * GS_THREADS, i0 = rank * GS_THREADS + threadIdx.x;
+    // element i of the three parts' concatenation, of vector m
+    auto at = [&](int m, int i) -> double2* {
+        const int f = (i >= n) + (i >= 2 * n);
+        return (f == 0 ? Y.y[0] : f == 1 ? Y.y[1] : Y.y[2]) + (size_t)m * n + (i - f * n);
+    };
+    // GS_B elements of a thread at a time, their loads in flight together; the
+    // first batch stays in registers between the product and the projection
+    double2 a0[GS_B], b0[GS_B];
+    auto load = [&](int i, double2* a, double2* b) {
+#pragma unroll
+        for (int u = 0; u < GS_B; ++u) {
+            a[u] = b[u] = make_double2(0.0, 0.0);
+            if (i + u * step < n3) {
+                b[u] = *at(j, i + u * step);
+                if (k >= 0) a[u] = *at(k, i + u * step);
+            }
+        }
+    };
+    load(i0, a0, b0);
     double2 c = make_double2(0.0, 0.0);
     if (k >= 0) {
         double2 s = make_double2(0.0, 0.0);
+        auto dot = [&](const double2* a, const double2* b) {
 #pragma unroll
-        for (int f = 0; f < 3; ++f) {
-            const double2 *xk = Y.y[f] + (size_t)k * n, *xj = Y.y[f] + (size_t)j * n;
-#pragma unroll 2
-            for (int i = i0; i < (int)n; i += step) {
-                const double2 a = xk[i], b = xj[i];
-                s.x += a.x * b.x + a.y * b.y;
-                s.y += a.x * b.y - a.y * b.x;
+            for (int u = 0; u < GS_B; ++u) {
+                s.x = fma(a[u].x, b[u].x, fma(a[u].y, b[u].y, s.x));
+                s.y = fma(a[u].x, b[u].y, fma(-a[u].y, b[u].x, s.y));
             }
+        };
+        dot(a0, b0);
+        for (int i = i0 + GS_B * step; i < n3; i += GS_B * step) {
+            double2 a[GS_B], b[GS_B];
+            load(i, a, b);
+            dot(a, b);
         }
-        s = cluster_sum(s, part, red);
-        const double nn = g.gsr[k];
-        c = make_double2(s.x / nn, s.y / nn);
+        c = cluster_sum(s, gs_inv(g)[k], sh);
     }
     const bool norm = j == k + 1;
     double2 s = make_double2(0.0, 0.0);
+    auto update = [&](int i, const double2* a, const double2* b) {
 #pragma unroll
-    for (int f = 0; f < 3; ++f) {
-        const double2* xk = Y.y[f] + (size_t)(k < 0 ? 0 : k) * n;
-        double2* xj = Y.y[f] + (size_t)j * n;
-#pragma unroll 2
-        for (int i = i0; i < (int)n; i += step) {
-            double2 b = xj[i];
-            if (k >= 0) {
-                const double2 a = xk[i];
-                b.x -= c.x * a.x - c.y * a.y;
-                b.y -= c.x * a.y + c.y * a.x;
-                xj[i] = b;
+        for (int u = 0; u < GS_B; ++u) {
+            double2 x = b[u];
+            if (k >= 0 && i + u * step < n3) {
+                x.x = fma(c.y, a[u].y, fma(-c.x, a[u].x, x.x));
+                x.y = fma(-c.y, a[u].x, fma(-c.x, a[u].y, x.y));
+                *at(j, i + u * step) = x;
             }
-            if (norm) s.x += b.x * b.x + b.y * b.y;
+            if (norm) s.x = fma(x.x, x.x, fma(x.y, x.y, s.x));
         }
+    };
+    update(i0, a0, b0);
+    for (int i = i0 + GS_B * step; i < n3; i += GS_B * step) {
+        double2 a[GS_B], b[GS_B];
+        load(i, a, b);
+        update(i, a, b);
     }
     if (norm) {
-        s = cluster_sum(s, part + 1, red);
-        if (cg::this_cluster().block_rank() == 0 && threadIdx.x == 0) g.gsr[j] = s.x;
+        __syncthreads();
+        s = cluster_sum(s, 1.0, sh);
+        if (rank == 0 && threadIdx.x == 0) {
+            gs_sq(g)[j] = s.x;
+            gs_inv(g)[j] = 1.0 / s.x;
+        }
     }
-    cg::this_cluster().sync();       // no CTA leaves while a peer may still read its part
 }
 
-// Every vector normalised and back in the state; its energy norm (the 1/4
-// included) recorded after the last CTA has read the squared norms.
+// Every vector normalised and back in the state, GS_EC members a CTA; the CTAs of
+// mode 0 record the energy norms (the 1/4 included).
 __global__ void __launch_bounds__(GS_THREADS) k_gs_scatter(GroupView g) {
-    const int Ny = g.ny, E = g.E, q = blockIdx.x;
+    extern __shared__ __align__(16) unsigned char sm[];
+    const int Ny = g.ny, E = g.E, q = blockIdx.x, e0 = blockIdx.y * GS_EC, ec = min(GS_EC, E - e0);
+    double* iw = (double*)sm;            // 1 / sqrt(w)
+    double* ir = iw + Ny;                // 1 / norm
+    for (int i = threadIdx.x; i < Ny + ec; i += blockDim.x) {
+        if (i < Ny) iw[i] = 1.0 / sqrt(g.ccw[i + 1]);
+        else {
+            const double r = sqrt(0.25 * gs_sq(g)[e0 + i - Ny]);
+            ir[i - Ny] = 1.0 / r;
+            if (q == 0) gs_norm(g)[e0 + i - Ny] = r;
+        }
+    }
+    __syncthreads();
     const GsParts Y = gs_parts(g);
     const size_t n = (size_t)g.nmodes * Ny;
     const double k1 = sqrt(1.0 / g.k2inv[q]);
-    for (int i = threadIdx.x; i < Ny * E; i += blockDim.x) {
-        const int y = i / E, e = i - y * E;
-        const double s = 1.0 / (sqrt(0.25 * g.gsr[e]) * sqrt(g.ccw[y + 1]));
-        const size_t o = (size_t)e * n + (size_t)q * Ny + y, h = ((size_t)q * Ny + y) * E + e;
+    for (int i = threadIdx.x; i < Ny * ec; i += blockDim.x) {
+        const int y = i / ec, el = i - y * ec;
+        const double s = iw[y] * ir[el], t = s * k1;
+        const size_t o = (size_t)(e0 + el) * n + (size_t)q * Ny + y, h = ((size_t)q * Ny + y) * E + e0 + el;
         const double2 a = Y.y[0][o], b = Y.y[2][o];
         g.v_t[h] = make_double2(a.x * s, a.y * s);
-        g.e_t[h] = make_double2(b.x * (s * k1), b.y * (s * k1));
+        g.e_t[h] = make_double2(b.x * t, b.y * t);
     }
-}
-__global__ void k_gs_norms(GroupView g) {
-    for (int e = threadIdx.x; e < g.E; e += blockDim.x) g.gsr[e] = sqrt(0.25 * g.gsr[e]);
 }
 
 int launch_lin_orthonormalize(const GroupView& g, cudaStream_t st) {
-    const size_t smem = 3 * (size_t)g.ny * GS_EC * sizeof(double2);
-    k_gs_gather<<<dim3(g.nmodes, (g.E + GS_EC - 1) / GS_EC), GS_THREADS, smem, st>>>(g);
+    const dim3 grid(g.nmodes, (g.E + GS_EC - 1) / GS_EC);
+    k_gs_gather<<<grid, GS_THREADS, 3 * (size_t)g.ny * GS_EC * sizeof(double2), st>>>(g);
     for (int k = -1; k < g.E - 1; ++k) k_gs_project<<<GS_CL * (k < 0 ? 1 : g.E - 1 - k), GS_THREADS, 0, st>>>(g, k);
-    k_gs_scatter<<<g.nmodes, GS_THREADS, 0, st>>>(g);
-    k_gs_norms<<<1, 64, 0, st>>>(g);
-    return g.E + 3;
+    k_gs_scatter<<<grid, GS_THREADS, (g.ny + GS_EC) * sizeof(double), st>>>(g);
+    return g.E + 2;
 }
 
 void set_attributes_linear() {

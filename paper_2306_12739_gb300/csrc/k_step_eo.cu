@@ -487,11 +487,12 @@ size_t helm_eo_smem_bytes(const GroupView& g) {
     return b > m ? b : m;
 }
 
-// the step-by-step stage in parity blocks: a DNS group (the operators of a
-// linear group need not be centro-symmetric) whose tiles fit
-bool step_eo_supported(const GroupView& g) {
-    return !g.lin && g.ny >= 3 && forcing_eo_smem_bytes(g) <= 227 * 1024 && helm_eo_smem_bytes(g) <= 227 * 1024;
+// the step-by-step stage in parity blocks: the tiles fit; by request only in DNS
+// groups (in a linear group the autotuner decides)
+bool step_eo_fits(const GroupView& g) {
+    return g.ny >= 3 && forcing_eo_smem_bytes(g) <= 227 * 1024 && helm_eo_smem_bytes(g) <= 227 * 1024;
 }
+bool step_eo_supported(const GroupView& g) { return !g.lin && step_eo_fits(g); }
 
 void launch_forcing_eo(const GroupView& g, int s, cudaStream_t st) {
     gt::Tile t = gt::tile_of(g.E, g.ny, g.nmodes);
