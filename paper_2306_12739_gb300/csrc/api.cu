@@ -41,6 +41,8 @@ struct HostGroup {
     dnsb::CnOps ops[2];
     std::vector<double> kxt, kzt, k2t, k2inv, twx, twz, opsdev[2], mopsdev[2], D1i, D2i;
     std::vector<double> ops64[2], D1EO64, D2EO64;   // FP64 path: the operators in parity blocks
+    std::vector<uint16_t> opsMM[2], D1MM, D2MM;     // fragments of the fused stage on mma.sync
+    int owner = -1;                                 // the block whose constant arrays this one uses (-1: its own)
     std::vector<float> kxtf, kztf, k2invf, twxf, twzf, opsf[2], opsfT[2], D1T, D2T, D2Tl, opsEO[2], D1EO, D2EO, D2lEO;
     std::vector<uint16_t> Atc, Htc[2], D2oz;
     std::vector<int> D2ozexp;
@@ -162,6 +164,10 @@ bool eo_candidate(const GroupView& v) { return (v.helm == 4 || v.helm == 0) && e
 bool step_eo_candidate(const GroupView& v) {
     return (v.helm == 0 || (v.helm == 1 && v.step_eo)) && dnsk::step_eo_fits(v);
 }
+// the fragments of the fused stage on mma.sync are wanted
+bool mma_candidate(const GroupView& v) {
+    return v.spec_mma && eo_candidate(v) && (v.helm == 0 || (v.spec_eo && v.spec_eoff));
+}
 bool eo_images(const GroupView& v) { return eo_candidate(v) || step_eo_candidate(v); }
 
 // Largest My at which DNS groups may take the FP32-accumulated tensor-core
@@ -223,6 +229,58 @@ void build_eo64_images(HostGroup& G, bool ops) {
     dnsk::spec_eo_image64(G.D2i.data(), v.ny, false, G.D2EO64.data());
 }
 
+// The fragments of the fused stage on mma.sync: M - I and P of every pair and step
+// length, D1, and D2's digits, from the FP64 matrices.
+// ops false: D1 and D2 only (the y-derivatives).
+void build_mma_images(HostGroup& G, bool ops, int nthreads) {
+    const GroupView& v = G.v;
+    const size_t nn = (size_t)v.ny * v.ny, mat = dnsk::spec_eo_mat_floats(v.ny), out = dnsk::spec_mma_mat_bytes(v.ny) / 2;
+    const size_t nmat = (size_t)v.npairs * 4;
+    for (int hi = 0; hi < 2 && ops; ++hi) {
+        G.opsMM[hi].resize(nmat * out);
+        auto work = [&](int t) {
+            std::vector<double> a(nn), eo(mat);
+            for (size_t blk = t; blk < nmat; blk += nthreads) {
+                memcpy(a.data(), &G.opsdev[hi][blk * nn], nn * sizeof(double));
+                if (blk % 2 == 0)
+                    for (int i = 0; i < v.ny; ++i) a[(size_t)i * v.ny + i] -= 1.0;
+                dnsk::spec_eo_image64(a.data(), v.ny, false, eo.data());
+                dnsk::spec_mma_image(eo.data(), v.ny, false, &G.opsMM[hi][blk * out]);
+            }
+        };
+        std::vector<std::thread> ts;
+        for (int t = 0; t < nthreads; ++t) ts.emplace_back(work, t);
+        for (auto& t : ts) t.join();
+    }
+    G.D1MM.resize(out);
+    dnsk::spec_mma_image(G.D1EO64.data(), v.ny, true, G.D1MM.data());
+    G.D2MM.resize(dnsk::spec_mma_d2_bytes(v.ny) / 2);
+    dnsk::spec_mma_d2_image(G.D2EO64.data(), v.ny, G.D2MM.data());
+}
+
+// Every constant array of a group's device view: the member blocks of a group
+// share them (f gets each pointer's address).
+template <typename F>
+void constants(GroupView& v, F f) {
+    const void** p[] = {
+        (const void**)&v.D1, (const void**)&v.D1i, (const void**)&v.D1EO64, (const void**)&v.D2EO64,
+        (const void**)&v.D1T, (const void**)&v.D2T, (const void**)&v.D2Tl, (const void**)&v.D1EO,
+        (const void**)&v.D2EO, (const void**)&v.D2lEO, &v.Atc, &v.D2oz, (const void**)&v.D2ozexp,
+        (const void**)&v.ccw, (const void**)&v.kxt, (const void**)&v.kzt, (const void**)&v.k2t, (const void**)&v.k2inv,
+        (const void**)&v.twx, (const void**)&v.twz, (const void**)&v.twxf, (const void**)&v.twzf,
+        (const void**)&v.kxtf, (const void**)&v.kztf, (const void**)&v.k2invf,
+        (const void**)&v.ops64[0], (const void**)&v.ops64[1], (const void**)&v.opsfT[0], (const void**)&v.opsfT[1],
+        &v.Htc[0], &v.Htc[1], (const void**)&v.opsEO[0], (const void**)&v.opsEO[1], (const void**)&v.mops[0],
+        (const void**)&v.mops[1], &v.opsMM[0], &v.opsMM[1], &v.D1MM, &v.D2MM};
+    for (const void** q : p) f(q);
+}
+// two member blocks want the same constant arrays
+bool same_constants(const GroupView& a, const GroupView& b) {
+    return ygemm_tc_candidate(a) == ygemm_tc_candidate(b) && ygemm_eo_candidate(a) == ygemm_eo_candidate(b) &&
+           eo_images(a) == eo_images(b) && helm_tc_candidate(a) == helm_tc_candidate(b) && a.d2tc == b.d2tc &&
+           mma_candidate(a) == mma_candidate(b);
+}
+
 size_t layout_group(dns_handle* h, HostGroup& G, size_t cur) {
     GroupView& v = G.v;
     G.slots.clear();
@@ -233,45 +291,53 @@ size_t layout_group(dns_handle* h, HostGroup& G, size_t cur) {
     };
     const size_t S = (size_t)v.nmodes * v.ny * v.E;  // complex elements of one spectral field
     const size_t nn = (size_t)v.ny * v.ny;
-    add((void**)&v.D1, sizeof(double) * v.my * v.my);
-    add((void**)&v.D1i, sizeof(double) * nn);
-    add((void**)&v.D1EO64, sizeof(double) * dnsk::spec_eo_mat_floats(v.ny));
-    add((void**)&v.D2EO64, sizeof(double) * dnsk::spec_eo_mat_floats(v.ny));
-    add((void**)&v.D1T, sizeof(float) * (size_t)v.ny * v.rp);
-    add((void**)&v.D2T, sizeof(float) * (size_t)v.ny * v.rp);
-    add((void**)&v.D2Tl, sizeof(float) * (size_t)v.ny * v.rp);
+    auto addc = [&](void** ptr, size_t bytes) { if (G.owner < 0) add(ptr, bytes); };
+    addc((void**)&v.D1, sizeof(double) * v.my * v.my);
+    addc((void**)&v.D1i, sizeof(double) * nn);
+    addc((void**)&v.D1EO64, sizeof(double) * dnsk::spec_eo_mat_floats(v.ny));
+    addc((void**)&v.D2EO64, sizeof(double) * dnsk::spec_eo_mat_floats(v.ny));
+    addc((void**)&v.D1T, sizeof(float) * (size_t)v.ny * v.rp);
+    addc((void**)&v.D2T, sizeof(float) * (size_t)v.ny * v.rp);
+    addc((void**)&v.D2Tl, sizeof(float) * (size_t)v.ny * v.rp);
     if (precision_mixed(h) && (eo_images(v) || ygemm_eo_candidate(v))) {
-        add((void**)&v.D1EO, sizeof(float) * dnsk::spec_eo_mat_floats(v.ny));
-        add((void**)&v.D2EO, sizeof(float) * dnsk::spec_eo_mat_floats(v.ny));
-        add((void**)&v.D2lEO, sizeof(float) * dnsk::spec_eo_mat_floats(v.ny));
+        addc((void**)&v.D1EO, sizeof(float) * dnsk::spec_eo_mat_floats(v.ny));
+        addc((void**)&v.D2EO, sizeof(float) * dnsk::spec_eo_mat_floats(v.ny));
+        addc((void**)&v.D2lEO, sizeof(float) * dnsk::spec_eo_mat_floats(v.ny));
     }
     add((void**)&v.status, 256);
-    if (ygemm_tc_candidate(v)) add((void**)&v.Atc, 3 * 128 * (size_t)v.kp * sizeof(uint16_t));
+    if (ygemm_tc_candidate(v)) addc((void**)&v.Atc, 3 * 128 * (size_t)v.kp * sizeof(uint16_t));
     if (v.d2tc) {
-        add((void**)&v.D2oz, dnsk::d2v_tc_image_bytes(v));
-        add((void**)&v.D2ozexp, 64 * sizeof(int));
+        addc((void**)&v.D2oz, dnsk::d2v_tc_image_bytes(v));
+        addc((void**)&v.D2ozexp, 64 * sizeof(int));
     }
-    add((void**)&v.ccw, sizeof(double) * v.my);
-    add((void**)&v.kxt, sizeof(double) * v.nkx);
-    add((void**)&v.kzt, sizeof(double) * v.nkz);
-    add((void**)&v.k2t, sizeof(double) * v.nmodes);
-    add((void**)&v.k2inv, sizeof(double) * v.nmodes);
-    add((void**)&v.twx, sizeof(double2) * v.mx);
-    add((void**)&v.twz, sizeof(double2) * v.mz);
-    add((void**)&v.twxf, sizeof(float2) * v.mx);
-    add((void**)&v.twzf, sizeof(float2) * v.mz);
-    add((void**)&v.kxtf, sizeof(float) * v.nkx);
-    add((void**)&v.kztf, sizeof(float) * v.nkz);
-    add((void**)&v.k2invf, sizeof(float) * v.nmodes);
+    if (precision_mixed(h) && mma_candidate(v))
+        for (int hi = 0; hi < 2; ++hi)
+            addc((void**)&v.opsMM[hi], (size_t)v.npairs * 4 * dnsk::spec_mma_mat_bytes(v.ny));
+    if (precision_mixed(h) && (mma_candidate(v) || ygemm_eo_candidate(v))) {
+        addc((void**)&v.D1MM, dnsk::spec_mma_mat_bytes(v.ny));
+        addc((void**)&v.D2MM, dnsk::spec_mma_d2_bytes(v.ny));
+    }
+    addc((void**)&v.ccw, sizeof(double) * v.my);
+    addc((void**)&v.kxt, sizeof(double) * v.nkx);
+    addc((void**)&v.kzt, sizeof(double) * v.nkz);
+    addc((void**)&v.k2t, sizeof(double) * v.nmodes);
+    addc((void**)&v.k2inv, sizeof(double) * v.nmodes);
+    addc((void**)&v.twx, sizeof(double2) * v.mx);
+    addc((void**)&v.twz, sizeof(double2) * v.mz);
+    addc((void**)&v.twxf, sizeof(float2) * v.mx);
+    addc((void**)&v.twzf, sizeof(float2) * v.mz);
+    addc((void**)&v.kxtf, sizeof(float) * v.nkx);
+    addc((void**)&v.kztf, sizeof(float) * v.nkz);
+    addc((void**)&v.k2invf, sizeof(float) * v.nmodes);
     for (int hi = 0; hi < 2; ++hi) {
         if (!precision_mixed(h))
-            add((void**)&v.ops64[hi], sizeof(double) * (size_t)v.npairs * 4 * dnsk::spec_eo_mat_floats(v.ny));
+            addc((void**)&v.ops64[hi], sizeof(double) * (size_t)v.npairs * 4 * dnsk::spec_eo_mat_floats(v.ny));
         if (precision_mixed(h)) {
-            add((void**)&v.opsfT[hi], sizeof(float) * (size_t)v.npairs * 4 * v.ny * v.rp);
-            if (helm_tc_candidate(v)) add((void**)&v.Htc[hi], (size_t)v.npairs * 2 * 3 * 64 * 2 * v.kp * sizeof(uint16_t));
-            if (eo_images(v)) add((void**)&v.opsEO[hi], sizeof(float) * (size_t)v.npairs * 4 * dnsk::spec_eo_mat_floats(v.ny));
+            addc((void**)&v.opsfT[hi], sizeof(float) * (size_t)v.npairs * 4 * v.ny * v.rp);
+            if (helm_tc_candidate(v)) addc((void**)&v.Htc[hi], (size_t)v.npairs * 2 * 3 * 64 * 2 * v.kp * sizeof(uint16_t));
+            if (eo_images(v)) addc((void**)&v.opsEO[hi], sizeof(float) * (size_t)v.npairs * 4 * dnsk::spec_eo_mat_floats(v.ny));
         }
-        add((void**)&v.mops[hi], sizeof(double) * (2 * nn + 3 * (size_t)v.ny + (size_t)v.ny * v.my));
+        addc((void**)&v.mops[hi], sizeof(double) * (2 * nn + 3 * (size_t)v.ny + (size_t)v.ny * v.my));
     }
     double2** st[] = {&v.v_t, &v.e_t, &v.v_s, &v.e_s, &v.mx1_v, &v.mx1_e, &v.Fv, &v.Fe, &v.Av, &v.Ae};
     for (auto p : st) add((void**)p, sizeof(double2) * S);
@@ -535,7 +601,10 @@ bool plane_variant_ok(bool mixed, const GroupView& v, int c) {
 //   against the cluster kernel on 128x97x128 x 4, 1099 -> 670 us in FP64;
 //   FP64 everywhere: 991 -> 548 us on 64x65x64 x 4, 154 -> 144 on 32x33x32 x 2; the single-CTA kernel spends its FP64 pipe on
 //   radix-2 to 4 passes and leaves SMs idle at few planes.
-bool plane_split_default(const GroupView& v, bool mixed) { return !mixed || v.mx == 128 || v.mz == 128; }
+bool plane_split_default(const GroupView& v, bool mixed) {
+    if (!mixed || v.mx == 128 || v.mz == 128) return true;
+    return false;
+}
 
 std::string tune_helm_key(const GroupView& v) {
     char b[128];
@@ -673,6 +742,7 @@ int choose_variants(dns_handle* h, const dns_config* cfg, GroupView& v, int gi) 
         v.spec_eoff = cfg->helm == 7 ? 1 : 0;
     }
     v.spec_minb = 2;
+    v.spec_mma = precision_mixed(h) && dnsk::spec_mma_supported(v) ? 1 : 0;
     // plane-stage kernel: single CTA per plane where it fits, a thread-block
     // cluster (distributed shared memory) where it does not; where both exist
     // the autotuner decides at bind time
@@ -775,20 +845,36 @@ int dns_create(const dns_config* cfg, void* cuda_stream, dns_handle** out) {
         m0 += d.members;
         HostGroup& G = h->groups[ig];
         if (b > 0) {
-            // a further block of the same group: same grid and operators (and nblk)
-            G = h->groups[ig0];
-            G.d = d;
-            G.v.E = d.members;
-            int rcv = choose_variants(h, cfg, G.v, gi);
+            // a further block of the same group: same grid and operators (and nblk),
+            // which it shares with the first
+            const HostGroup& G0 = h->groups[ig0];
+            GroupView vb = G0.v;
+            vb.E = d.members;
+            vb.helm = vb.ygemm = vb.plane = 0;
+            int rcv = choose_variants(h, cfg, vb, gi);
             if (rcv) return rcv;
-            if (ygemm_tc_candidate(G.v) && G.Atc.empty()) G.Atc = dnsk::yderiv_tc_a_image(G.D1i, G.D2i, G.v.ny, G.v.kp);
-            if (G.v.d2tc && G.D2oz.empty()) dnsk::d2v_tc_image(G.D2i, G.v.ny, G.v.kp, G.D2oz, G.D2ozexp);
-            if (precision_mixed(h) && ((eo_images(G.v) && G.opsEO[0].empty()) ||
-                                       (ygemm_eo_candidate(G.v) && G.D1EO.empty())))
-                build_eo_images(G, eo_images(G.v));
-            if (precision_mixed(h) && helm_tc_candidate(G.v) && G.Htc[0].empty())
-                for (int hi = 0; hi < 2; ++hi)
-                    G.Htc[hi] = dnsk::helm_tc_a_images(G.opsdev[hi], G.v.npairs, G.v.ny, G.v.kp);
+            if (same_constants(G0.v, vb)) {
+                G.owner = ig0;
+                G.grid = G0.grid;
+                G.kxt = G0.kxt; G.kzt = G0.kzt; G.k2t = G0.k2t; G.k2inv = G0.k2inv;
+                G.D1i = G0.D1i; G.D2i = G0.D2i;
+            } else {
+                G = G0;
+                if (ygemm_tc_candidate(vb) && G.Atc.empty()) G.Atc = dnsk::yderiv_tc_a_image(G.D1i, G.D2i, vb.ny, vb.kp);
+                if (vb.d2tc && G.D2oz.empty()) dnsk::d2v_tc_image(G.D2i, vb.ny, vb.kp, G.D2oz, G.D2ozexp);
+                G.v = vb;
+                if (precision_mixed(h) && ((eo_images(vb) && G.opsEO[0].empty()) ||
+                                           (ygemm_eo_candidate(vb) && G.D1EO.empty())))
+                    build_eo_images(G, eo_images(vb));
+                if (precision_mixed(h) && helm_tc_candidate(vb) && G.Htc[0].empty())
+                    for (int hi = 0; hi < 2; ++hi)
+                        G.Htc[hi] = dnsk::helm_tc_a_images(G.opsdev[hi], vb.npairs, vb.ny, vb.kp);
+                if (precision_mixed(h) && ((mma_candidate(vb) && G.opsMM[0].empty()) ||
+                                           (ygemm_eo_candidate(vb) && G.D1MM.empty())))
+                    build_mma_images(G, mma_candidate(vb), nthreads);
+            }
+            G.d = d;
+            G.v = vb;
             cur = layout_group(h, G, cur);
             continue;
         }
@@ -922,6 +1008,8 @@ int dns_create(const dns_config* cfg, void* cuda_stream, dns_handle** out) {
         if (precision_mixed(h) && helm_tc_candidate(v))
             for (int hi = 0; hi < 2; ++hi) G.Htc[hi] = dnsk::helm_tc_a_images(G.opsdev[hi], v.npairs, v.ny, v.kp);
         build_eo64_images(G, !precision_mixed(h));
+        if (precision_mixed(h) && (mma_candidate(v) || ygemm_eo_candidate(v)))
+            build_mma_images(G, mma_candidate(v), nthreads);
         if (!lin) G.twx = dnsb::twiddles(d.mx);
         G.twz = dnsb::twiddles(d.mz);
         G.twxf.assign(G.twx.begin(), G.twx.end());
@@ -985,6 +1073,7 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
     dnsk::set_attributes_helm_tc();
     dnsk::set_attributes_linear();
     dnsk::set_attributes_spec();
+    dnsk::set_attributes_spec_mma();
     dnsk::set_attributes_step_eo();
     dnsk::set_attributes_step64();
     dnsk::set_attributes_d2v_tc();
@@ -1000,6 +1089,12 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
     for (auto& G : h->groups) {
         for (auto& s : G.slots) *s.first = h->ws + s.second.off;
         GroupView& v = G.v;
+        if (G.owner >= 0) {
+            std::vector<const void*> from;
+            constants(h->groups[G.owner].v, [&](const void** q) { from.push_back(*q); });
+            size_t i = 0;
+            constants(v, [&](const void** q) { *q = from[i++]; });
+        }
         if (!precision_mixed(h)) v.P5d = (double2*)v.P5;
         struct Up { const void* dst; const void* src; size_t bytes; };
         const Up ups[] = {
@@ -1036,11 +1131,15 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
             {v.D2EO, G.D2EO.data(), G.D2EO.size() * 4},
             {v.D2lEO, G.D2lEO.data(), G.D2lEO.size() * 4},
             {v.D2ozexp, G.D2ozexp.data(), G.D2ozexp.size() * 4},
+            {v.opsMM[0], G.opsMM[0].data(), G.opsMM[0].size() * 2},
+            {v.opsMM[1], G.opsMM[1].data(), G.opsMM[1].size() * 2},
+            {v.D1MM, G.D1MM.data(), G.D1MM.size() * 2},
+            {v.D2MM, G.D2MM.data(), G.D2MM.size() * 2},
             {v.mops[0], G.mopsdev[0].data(), G.mopsdev[0].size() * 8},
             {v.mops[1], G.mopsdev[1].data(), G.mopsdev[1].size() * 8},
         };
         for (const auto& u : ups) {
-            if (u.bytes == 0 || u.dst == nullptr) continue;
+            if (u.bytes == 0 || u.dst == nullptr || G.owner >= 0) continue;
             rc = check(h, cudaMemcpyAsync((void*)u.dst, u.src, u.bytes, cudaMemcpyHostToDevice, st), "upload operators");
             if (rc) return rc;
         }

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <cstddef>
+#include <cstdint>
 #include "common.cuh"
 
 namespace dnsk {
@@ -70,6 +71,10 @@ struct GroupView {
     const float* D1EO;      // D1 in parity blocks
     const float* D2EO;      // D2 in parity blocks and its residual D2 - (double) D2EO
     const float* D2lEO;
+    int spec_mma;         // fused stage in parity blocks with spec_eoff: 1 = products on mma.sync (k_spec_mma.cu)
+    const void* opsMM[2]; // its operator fragments, per h index: [npairs][4] matrices (M - I, P of v and eta)
+    const void* D1MM;     // ... of D1, and D2's digits
+    const void* D2MM;
     int spec_ec;          // fused stage: members per CTA (0 = up to 8), set by the autotuner
     int yd_cap;           // register-tiled y-derivatives: first column-tile cap (0 = 64, or 32 above
                           //    Ny = 96), halved while the grid is short of 3 CTAs per SM; autotuned
@@ -192,6 +197,17 @@ void spec_eo_image64(const double* A, int ny, bool anti, double* out);
 size_t spec_smem_bytes(const GroupView& g);
 void launch_spec(const GroupView& g, int s, cudaStream_t st);
 void set_attributes_spec();
+// that stage with its products on mma.sync (k_spec_mma.cu): images from a matrix
+// in parity blocks (spec_eo_image64)
+bool spec_mma_supported(const GroupView& g);
+size_t spec_mma_mat_bytes(int ny);
+size_t spec_mma_d2_bytes(int ny);
+void spec_mma_image(const double* eo, int ny, bool anti, uint16_t* out);
+void spec_mma_d2_image(const double* eo, int ny, uint16_t* out);
+void launch_spec_mma(const GroupView& g, int s, cudaStream_t st);
+void launch_mma_derivs(const GroupView& g, cudaStream_t st);
+void launch_yderiv_mma(const GroupView& g, const double2* v, const double2* e, cudaStream_t st, int sprev);
+void set_attributes_spec_mma();
 // the step-by-step y-derivatives, forcing and implicit apply in parity blocks (k_step_eo.cu)
 bool yderiv_eo_supported(const GroupView& g);
 size_t yderiv_eo_smem_bytes(const GroupView& g);

@@ -516,6 +516,10 @@ size_t yderiv_eo_smem_bytes(const GroupView& g) {
 bool yderiv_eo_supported(const GroupView& g) { return g.ny >= 3 && yderiv_eo_smem_bytes(g) <= 227 * 1024; }
 
 void launch_yderiv_eo(const GroupView& g, const double2* v, const double2* e, cudaStream_t st, int sprev) {
+    if (g.D1MM != nullptr && g.D2MM != nullptr) {
+        launch_yderiv_mma(g, v, e, st, sprev);
+        return;
+    }
     const gt::Tile t = sto::yde_tile(g.E, g.ny, g.nmodes, g.yd_cap);
     dim3 grid((g.nmodes + t.QT - 1) / t.QT, (g.E + t.EBT - 1) / t.EBT);
     grid.y += mean_finish_extra_rows(g, grid.x, sprev);

@@ -110,6 +110,75 @@ __device__ __forceinline__ void mean_finish(const GroupView& g, int s, int e, un
     if (threadIdx.x == 0) g.gamma[e] = gam;
 }
 
+// Finish of a member's mean-flow update after its last row CTA (see
+// mean_finish): gamma, the profiles, the RK accumulators of <uv>, <wv>.  The
+// pre-gamma rows dU, dW were written by other CTAs of this launch: they are
+// read through L2.
+__device__ inline void finish_member(const GroupView& g, int s, int e, unsigned char* sm) {
+    const int Ny = g.ny, My = g.my;
+    double* red = (double*)sm;
+    const int hi = (s == 0) ? 0 : 1;
+    const double* Ug = g.mops[hi] + 2 * (size_t)Ny * Ny + 2 * (size_t)Ny;
+    const double* Un = g.dU + (size_t)e * My;
+    const double* Wn = g.dW + (size_t)e * My;
+    const double* Ut = g.U_t + (size_t)e * My;
+    const double* Wt = g.W_t + (size_t)e * My;
+    double gam = 0.0;
+    if (g.flow == 1) {
+        double fl = 0.0, fg = 0.0;
+        for (int j = threadIdx.x; j < My; j += blockDim.x)
+            fl += g.ccw[j] * ((j > 0 && j < My - 1) ? __ldcg(Un + j) : Ut[j]);
+        for (int i = threadIdx.x; i < Ny; i += blockDim.x) fg += g.ccw[i + 1] * Ug[i];
+        fl = block_sum(fl, red);
+        fg = block_sum(fg, red);
+        gam = (g.bulk_flux - fl) / fg;
+    }
+    double* Uo = (s == 2) ? (g.U_t + (size_t)e * My) : (g.U_s + (size_t)e * My);
+    double* Wo = (s == 2) ? (g.W_t + (size_t)e * My) : (g.W_s + (size_t)e * My);
+    const double u0 = Ut[0], u1 = Ut[My - 1], w0 = Wt[0], w1 = Wt[My - 1];
+    __syncthreads();
+    for (int j = threadIdx.x; j < My; j += blockDim.x) {
+        const bool wall = (j == 0 || j == My - 1);
+        Uo[j] = wall ? (j == 0 ? u0 : u1) : __ldcg(Un + j) + gam * Ug[j - 1];
+        Wo[j] = wall ? (j == 0 ? w0 : w1) : __ldcg(Wn + j);
+        const size_t o = (size_t)e * My + j;
+        if (s == 0) {
+            g.AU[o] = g.uv[o];
+            g.AW[o] = g.wv[o];
+        } else if (s == 1) {
+            g.AU[o] = (1.0 / 6.0) * g.AU[o] + (4.0 / 6.0) * g.uv[o];
+            g.AW[o] = (1.0 / 6.0) * g.AW[o] + (4.0 / 6.0) * g.wv[o];
+        }
+    }
+    if (threadIdx.x == 0) g.gamma[e] = gam;
+    // the step is complete: the next step draws new noise
+    if (s == 2 && g.fn > 0 && e == 0 && threadIdx.x == 0) *g.fstep += 1ULL;
+}
+
+// mean-row CTAs of a member in a launch of `threads` threads per CTA
+__host__ __device__ inline int mean_ctas_per_member(const GroupView& g, int threads) {
+    return (g.ny + threads / 32 - 1) / (threads / 32);
+}
+
+// Rows of the mean-flow update (one warp per interior row), then the member's
+// finish by whichever of its row CTAs completes last (a counter per member,
+// reset by that CTA for the next launch).
+__device__ inline void mean_cta(const GroupView& g, int s, int b, unsigned char* sm) {
+    const int E = g.E, per = mean_ctas_per_member(g, blockDim.x);
+    const int e = b % E, r = b / E;
+    if (!DNS_CK(g.status, r < per, CK_SPEC, b)) return;
+    mean_rows(g, s, e, r * (blockDim.x / 32), sm);
+    __shared__ int last;
+    __threadfence();        // this CTA's rows are visible device-wide before it counts itself
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&g.mcnt[e], 1) == per - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    finish_member(g, s, e, sm);
+    if (threadIdx.x == 0) g.mcnt[e] = 0;
+}
+
 // The finish of sub-steps 1 and 2 rides on the next sub-step's y-derivative
 // launch (it is independent of it and done before the plane stage reads the
 // profiles): grid rows gy0 and beyond of that 2-D launch hold one CTA per
