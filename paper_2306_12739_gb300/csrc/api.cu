@@ -600,10 +600,16 @@ bool plane_variant_ok(bool mixed, const GroupView& v, int c) {
 //   128-point grids, where a plane does not fit one SM: 404 -> 153 us a launch
 //   against the cluster kernel on 128x97x128 x 4, 1099 -> 670 us in FP64;
 //   FP64 everywhere: 991 -> 548 us on 64x65x64 x 4, 154 -> 144 on 32x33x32 x 2; the single-CTA kernel spends its FP64 pipe on
-//   radix-2 to 4 passes and leaves SMs idle at few planes.
+//   radix-2 to 4 passes and leaves SMs idle at few planes;
+//   large mixed advective groups (1.5 M interior points over all members, both
+//   lengths 32 and more), whose launches fill the chip several times, so that the
+//   fewer instructions count and the two extra launches do not: whole steps of
+//   32x49x32 x 64 496 -> 411 us, x 32 271 -> 240, x 16 169 -> 177; 64x65x64 x 8
+//   331 -> 324, x 4 174 -> 187; in the rotational form (fewer transforms) 282 -> 298.
 bool plane_split_default(const GroupView& v, bool mixed) {
     if (!mixed || v.mx == 128 || v.mz == 128) return true;
-    return false;
+    const double points = (double)v.ny * v.E * v.nblk * v.mx * v.mz;
+    return !v.rot && v.mx >= 32 && v.mz >= 32 && points >= 1.5e6;
 }
 
 std::string tune_helm_key(const GroupView& v) {
