@@ -25,7 +25,9 @@
 //     vectors: one launch per vector k projects x_k out of every later vector, a
 //     thread-block cluster each.
 #include "dns_internal.hpp"
+#include "dft.cuh"
 #include "eo.cuh"
+#include "pairs.cuh"
 #include <cooperative_groups.h>
 
 namespace cg = cooperative_groups;
@@ -33,16 +35,6 @@ namespace cg = cooperative_groups;
 namespace dnsk {
 
 constexpr int GS_THREADS = 256;
-
-// threads of the plane stage for transforms of length MZ: one per butterfly of
-// the widest stage over the nine lines (at most 320)
-__host__ __device__ constexpr int lin_threads(int MZ) {
-    int nb = 0;
-    for (int s = 0; s < ct_stages(MZ); ++s) nb = MZ / ct_radix(MZ, s) > nb ? MZ / ct_radix(MZ, s) : nb;
-    int t = 9 * nb;
-    t = t > 320 ? 320 : t;
-    return (t + 31) / 32 * 32;
-}
 
 template <typename T> struct LinTab;
 template <> struct LinTab<double> {
@@ -58,115 +50,187 @@ template <> struct LinTab<float> {
     static __device__ __forceinline__ const float* kz(const GroupView& g) { return g.kztf; }
 };
 
-template <typename T>
-size_t lin_plane_smem_bytes(int mz) {
-    return 2 * 9 * (size_t)mz * sizeof(typename C2<T>::type);
-}
+using namespace prs;
 
-// i * (a x + b y) for complex x, y and real a, b
-template <typename C, typename T>
-__device__ __forceinline__ C i_lin2(T a, C x, T b, C y) {
-    C r;
-    r.x = -(a * x.y + b * y.y);
-    r.y = a * x.x + b * y.x;
-    return r;
-}
+// The plane stage: one CTA per interior plane and NV vectors, one warp per field
+// (u, v, w, then their y- and z-derivatives), 32 / H = NV transforms of H lanes in
+// a warp.  A transform of Mz = N1 N2 points is a four-step one inside its lanes (a
+// lane does the residues 2 j and 2 j + 1 modulo N2 as a pair, then N2-point DFTs
+// whose two halves are the rows p and p + Mz/2), so only the products between the
+// inverse and the forward transforms need the CTA together.  61 planes x 45 vectors
+// of 64 points: 16.7 us a launch with a Stockham transform of the nine lines of one
+// vector per CTA, a barrier per radix-4 pass.
+template <int MZ> struct LinCfg {
+    static constexpr int N1 = dft::Split<MZ>::N1, N2 = dft::Split<MZ>::N2, H = N2 / 2, HP = MZ / 2;
+    static constexpr int NV = 32 / H;                         // vectors of a CTA
+    static constexpr int NQ = (N1 + H - 1) / H;               // N2-point tasks per lane
+    static constexpr int KZ = (MZ - 1) / 3;
+    static constexpr int XS = H + 1;                          // rows of the exchange (complex pairs)
+    // a transform's storage: its exchange, then its points; for H = 4 two transforms
+    // share an eight-lane access and lie four 16-byte banks apart
+    static constexpr int R0 = N1 * XS > HP ? N1 * XS : HP;
+    static constexpr int RS = H == 4 ? R0 + ((4 - R0 % 8) + 8) % 8 : R0;
+};
+constexpr int LIN_THREADS = 9 * 32;
 
-template <typename C, typename T>
-__device__ __forceinline__ C axpy3(T a, C x, T b, C y, T c, C z) {
-    C r;
-    r.x = a * x.x + b * y.x + c * z.x;
-    r.y = a * x.y + b * y.y + c * z.y;
-    return r;
+template <typename T, int MZ>
+size_t lin_plane_smem_bytes() {
+    typedef LinCfg<MZ> K;
+    return sizeof(Pc<T>) * (9 * K::NV * K::RS + K::N1 * K::H);
 }
 
 template <typename T, int MZ>
-__global__ void __launch_bounds__(lin_threads(MZ)) k_lin_plane(GroupView g) {
-    typedef typename C2<T>::type C;
+__global__ void __launch_bounds__(LIN_THREADS, sizeof(T) == 4 ? 2 : 1) k_lin_plane(GroupView g) {
+    typedef LinCfg<MZ> K;
+    constexpr int N1 = K::N1, N2 = K::N2, H = K::H, HP = K::HP, NV = K::NV, KZ = K::KZ, XS = K::XS, RS = K::RS;
+    struct Cv { T x, y; };
     extern __shared__ __align__(16) unsigned char sm[];
-    const int y = blockIdx.x, e = blockIdx.y;
-    constexpr int Mz = MZ;
-    const int Ny = g.ny, E = g.E, NM = g.nmodes, Kz = g.kz;
-    C* b0 = (C*)sm;
-    C* b1 = b0 + 9 * Mz;
-    const bool adjoint = *g.dir != 0;
-    const size_t fs = (size_t)Ny * E * NM;
-    const C* P = (const C*)g.P5 + ((size_t)y * E + e) * NM;
+    Pc<T>* X = (Pc<T>*)sm;                                     // [field][vector][RS]
+    Pc<T>* tw = X + 9 * NV * RS;                               // [k1][j]: the residue pair (2 j, 2 j + 1)
+    const int y = blockIdx.x, e0 = blockIdx.y * NV, E = g.E, NM = g.nmodes;
+    const int tid = threadIdx.x, lane = tid & 31, f = tid >> 5, j = lane % H, vec = lane / H;
+    const bool live = e0 + vec < E;
+    const size_t fs = (size_t)g.ny * E * NM;
+    for (int i = tid; i < N1 * H; i += LIN_THREADS) {
+        const int k1 = i / H, r = i - k1 * H;
+        const auto a = LinTab<T>::tw(g)[2 * r * k1], b = LinTab<T>::tw(g)[(2 * r + 1) * k1];
+        tw[i] = {pr((T)a.x, (T)b.x), pr((T)a.y, (T)b.y)};
+    }
     const T kx = (T)g.kxt[0];
-    const T* kzt = LinTab<T>::kz(g);
-    const T* k2i = LinTab<T>::k2i(g);
-    for (int i = threadIdx.x; i < 9 * Mz; i += blockDim.x) b0[i] = czero<C>();
-    __syncthreads();
-    // zero-padded spectral lines: u, v, w | d_y u, d_y v, d_y w | d_z u, d_z v, d_z w
-    for (int q = threadIdx.x; q < NM; q += blockDim.x) {
-        const int m = q - Kz, pos = m >= 0 ? m : m + Mz;
-        const C v = P[q], dv = P[fs + q], d2v = P[2 * fs + q], et = P[3 * fs + q], de = P[4 * fs + q];
-        const T kz = kzt[q], ki = k2i[q];
-        // u = i (kx Dv - kz eta) / k^2, w = i (kz Dv + kx eta) / k^2
-        const C u = cscale(i_lin2(kx, dv, -kz, et), ki);
-        const C w = cscale(i_lin2(kz, dv, kx, et), ki);
-        const C uy = cscale(i_lin2(kx, d2v, -kz, de), ki);
-        const C wy = cscale(i_lin2(kz, d2v, kx, de), ki);
-        b0[0 * Mz + pos] = u;
-        b0[1 * Mz + pos] = v;
-        b0[2 * Mz + pos] = w;
-        b0[3 * Mz + pos] = uy;
-        b0[4 * Mz + pos] = dv;
-        b0[5 * Mz + pos] = wy;
-        b0[6 * Mz + pos] = cscale(cmuli(u), kz);
-        b0[7 * Mz + pos] = cscale(cmuli(v), kz);
-        b0[8 * Mz + pos] = cscale(cmuli(w), kz);
+    Pc<T>* L = X + (f * NV + vec) * RS;
+
+    // ---- field f = 3 kind + comp: u_comp, d_y u_comp (kind 1), d_z u_comp (2), with
+    // u = i (kx Dv - kz eta) / k^2, w = i (kz Dv + kx eta) / k^2 (d_y: D2v, D eta)
+    const int kind = f / 3, comp = f - 3 * kind;
+    Pc<T> v[N1];
+    {
+        const Cv* P = (const Cv*)g.P5 + ((size_t)y * E + e0 + vec) * NM;
+        const Cv* A = P + (comp == 1 ? (kind == 1 ? 1 : 0) : (kind == 1 ? 2 : 1)) * fs;
+        const Cv* B = P + (kind == 1 ? 4 : 3) * fs;
+        const T* kzt = LinTab<T>::kz(g);
+        const T* k2i = LinTab<T>::k2i(g);
+#pragma unroll
+        for (int n1 = 0; n1 < N1; ++n1) {
+            v[n1] = {dup((T)0), dup((T)0)};
+            const int z0 = N2 * n1;
+            if (z0 > KZ && z0 + N2 - 1 < MZ - KZ) continue;      // wholly padding
+            Cv c[2];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int z = z0 + 2 * j + r;
+                const bool lo = z <= KZ;
+                c[r] = {(T)0, (T)0};
+                if (!live || !(lo || z >= MZ - KZ)) continue;
+                const int q = lo ? z + KZ : z - MZ + KZ;
+                const T kz = kzt[q];
+                Cv a = A[q];
+                if (comp != 1) {
+                    const Cv b = B[q];
+                    const T ki = k2i[q], ka = comp == 0 ? kx : kz, kb = comp == 0 ? -kz : kx;
+                    a = {-((ka * a.y + kb * b.y) * ki), (ka * a.x + kb * b.x) * ki};
+                }
+                c[r] = kind == 2 ? Cv{-kz * a.y, kz * a.x} : a;
+            }
+            v[n1] = {pr(c[0].x, c[1].x), pr(c[0].y, c[1].y)};
+        }
+    }
+    pdft_padded<N1, +1>(v);
+    __syncthreads();                                             // the twiddles
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) stp(L + k1 * XS + j, k1 == 0 ? v[0] : pmul<true>(v[k1], ldp(tw + k1 * H + j)));
+    __syncwarp();
+    Pc<T> o[K::NQ][H];
+#pragma unroll
+    for (int q = 0; q < K::NQ; ++q) {
+        const int k1 = j + H * q;
+        if (K::NQ * H > N1 && k1 >= N1) continue;
+#pragma unroll
+        for (int i = 0; i < H; ++i) o[q][i] = ldp(L + k1 * XS + i);
+        dft_dit<N2, +1>(o[q]);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < K::NQ; ++q) {
+        const int k1 = j + H * q;
+        if (K::NQ * H > N1 && k1 >= N1) continue;
+#pragma unroll
+        for (int k = 0; k < H; ++k) stp(L + k1 + N1 * k, o[q][k]);
     }
     __syncthreads();
-    C* ph = fft_lines_ct<C, +1, MZ, 9>(b0, b1, LinTab<T>::tw(g));
-    // products at every z (one thread reads the nine values at z and writes the
-    // three results there)
-    const T* B = LinTab<T>::base(g) + (size_t)y * Mz;
-    const size_t bs = (size_t)Ny * Mz;
-    for (int z = threadIdx.x; z < Mz; z += blockDim.x) {
-        C a[9];
+
+    // ---- products at the rows p and p + Mz/2, over the lines of u, v, w
+    const bool adjoint = *g.dir != 0;
+    const size_t bs = (size_t)g.ny * MZ;
+    for (int i = tid; i < NV * HP; i += LIN_THREADS) {
+        const int ve = i / HP, p = i - ve * HP;
+        const T* B = LinTab<T>::base(g) + (size_t)y * MZ + p;
+        Pc<T> a[9];
 #pragma unroll
-        for (int f = 0; f < 9; ++f) a[f] = ph[f * Mz + z];
-        const T U = B[z], V = B[bs + z], W = B[2 * bs + z];
-        const T By[3] = {B[3 * bs + z], B[4 * bs + z], B[5 * bs + z]};
-        const T Bz[3] = {B[6 * bs + z], B[7 * bs + z], B[8 * bs + z]};
-        C N[3];
+        for (int c = 0; c < 9; ++c) a[c] = ldp(X + (c * NV + ve) * RS + p);
+        auto base = [&](int c) { return pr(B[c * bs], B[c * bs + HP]); };
+        const Pr<T> U = base(0) * dup(kx), V = base(1), W = base(2);
+        Pr<T> By[3], Bz[3];
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            // (B . grad) a_i = i kx U a_i + V d_y a_i + W d_z a_i
-            C adv = cscale(cmuli(a[i]), kx * U);
-            adv.x += V * a[3 + i].x + W * a[6 + i].x;
-            adv.y += V * a[3 + i].y + W * a[6 + i].y;
+        for (int c = 0; c < 3; ++c) { By[c] = base(3 + c); Bz[c] = base(6 + c); }
+        Pc<T> N[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            // (B . grad) a_c = i kx U a_c + V d_y a_c + W d_z a_c
+            const Pc<T> adv = {pfma(V, a[3 + c].x, W * a[6 + c].x) - U * a[c].y,
+                               pfma(V, a[3 + c].y, pfma(W, a[6 + c].y, U * a[c].x))};
             if (!adjoint) {
-                N[i].x = adv.x + a[1].x * By[i] + a[2].x * Bz[i];
-                N[i].y = adv.y + a[1].y * By[i] + a[2].y * Bz[i];
-            } else if (i == 0) {
-                N[i].x = -adv.x;
-                N[i].y = -adv.y;
+                N[c] = {pfma(a[1].x, By[c], pfma(a[2].x, Bz[c], adv.x)), pfma(a[1].y, By[c], pfma(a[2].y, Bz[c], adv.y))};
+            } else if (c == 0) {
+                N[c] = {pneg(adv.x), pneg(adv.y)};
             } else {
-                const C t = (i == 1) ? axpy3(By[0], a[0], By[1], a[1], By[2], a[2])
-                                     : axpy3(Bz[0], a[0], Bz[1], a[1], Bz[2], a[2]);
-                N[i].x = t.x - adv.x;
-                N[i].y = t.y - adv.y;
+                const Pr<T>* G = c == 1 ? By : Bz;
+                N[c] = {pfma(G[0], a[0].x, pfma(G[1], a[1].x, G[2] * a[2].x)) - adv.x,
+                        pfma(G[0], a[0].y, pfma(G[1], a[1].y, G[2] * a[2].y)) - adv.y};
             }
         }
 #pragma unroll
-        for (int i = 0; i < 3; ++i) ph[i * Mz + z] = N[i];
+        for (int c = 0; c < 3; ++c) stp(X + (c * NV + ve) * RS + p, N[c]);
     }
     __syncthreads();
-    C* out = fft_lines_ct<C, -1, MZ, 3>(ph, ph == b0 ? b1 : b0, LinTab<T>::tw(g));
-    // keep |m| <= Kz; the forward transform carries 1/Mz
-    const T sc = (T)(1.0 / (double)Mz);
-    C* N3 = (C*)g.N3 + ((size_t)y * E + e) * NM;
-    for (int i = threadIdx.x; i < 3 * NM; i += blockDim.x) {
-        const int f = i / NM, q = i - f * NM, m = q - Kz, pos = m >= 0 ? m : m + Mz;
-        N3[(size_t)f * fs + q] = cscale(out[f * Mz + pos], sc);
+
+    // ---- forward transforms, kept modes, 1 / Mz
+    if (f >= 3) return;
+#pragma unroll
+    for (int q = 0; q < K::NQ; ++q) {
+        const int k1 = j + H * q;
+        if (K::NQ * H > N1 && k1 >= N1) continue;
+#pragma unroll
+        for (int k = 0; k < H; ++k) o[q][k] = ldp(L + k1 + N1 * k);
+        dft_dif<N2, -1>(o[q]);
     }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < K::NQ; ++q) {
+        const int k1 = j + H * q;
+        if (K::NQ * H > N1 && k1 >= N1) continue;
+#pragma unroll
+        for (int i = 0; i < H; ++i) stp(L + k1 * XS + i, pmul<false>(o[q][i], ldp(tw + k1 * H + i)));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) v[k1] = ldp(L + k1 * XS + j);
+    Pdft<N1, -1, T>::run(v);
+    if (!live) return;
+    Cv* out = (Cv*)g.N3 + (size_t)f * fs + ((size_t)y * E + e0 + vec) * NM;
+    const T sc = (T)(1.0 / (double)MZ);
+#pragma unroll
+    for (int k2 = 0; k2 < N1; ++k2)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int m = 2 * j + r + N2 * k2, q = m <= KZ ? m + KZ : (m >= MZ - KZ ? m - MZ + KZ : -1);
+            if (q >= 0) out[q] = {(r ? v[k2].x.b : v[k2].x.a) * sc, (r ? v[k2].y.b : v[k2].y.a) * sc};
+        }
 }
 
 template <typename T, int MZ>
 void launch_lin_plane_t(const GroupView& g, cudaStream_t st) {
-    k_lin_plane<T, MZ><<<dim3(g.ny, g.E), lin_threads(MZ), lin_plane_smem_bytes<T>(MZ), st>>>(g);
+    constexpr int NV = LinCfg<MZ>::NV;
+    k_lin_plane<T, MZ><<<dim3(g.ny, (g.E + NV - 1) / NV), LIN_THREADS, lin_plane_smem_bytes<T, MZ>(), st>>>(g);
 }
 
 template <typename T>
@@ -425,7 +489,9 @@ int launch_lin_orthonormalize(const GroupView& g, cudaStream_t st) {
 
 void set_attributes_linear() {
     allow_max_dynamic_smem(k_gs_gather);
-    // the plane stage needs at most 2 x 9 x 128 x 16 B = 36 KB, below the default limit
+#define DNS_CASE(a) allow_max_dynamic_smem(k_lin_plane<float, a>); allow_max_dynamic_smem(k_lin_plane<double, a>);
+    DNS_CASE(16) DNS_CASE(32) DNS_CASE(48) DNS_CASE(64) DNS_CASE(128)
+#undef DNS_CASE
 }
 
 }  // namespace dnsk

@@ -218,7 +218,7 @@ __device__ __forceinline__ void two_sum(float& h, float& l, float b) {
 template <int KT>
 __device__ __forceinline__ void d2_product(const GroupView& g, const bf* dig, const Shape& S, const Place& w, Out& out) {
     const unsigned at = su32(dig + (8 * w.nt + (w.lane & 7)) * S.CS + ((w.lane >> 3) & 1) * 8 + (w.lane >> 4) * S.VP);
-#pragma unroll
+#pragma unroll 1
     for (int blk = 0; blk < 2; ++blk) {
         const uint4* A = (const uint4*)g.D2MM + (size_t)blk * KT * KT * oz::NDIG * 32;
         float acc[oz::NLEV][4];
@@ -247,7 +247,8 @@ __device__ __forceinline__ void d2_product(const GroupView& g, const bf* dig, co
             float h = acc[0][i], l = __fadd_rn(__fadd_rn(acc[5][i], acc[4][i]), acc[3][i]);
             two_sum(h, l, acc[1][i]);
             two_sum(h, l, acc[2][i]);
-            (blk ? out.o : out.e)[i] = __fadd_rn(h, l);
+            if (!blk) out.e[i] = __fadd_rn(h, l);
+            else out.o[i] = __fadd_rn(h, l);
         }
     }
 }
@@ -386,23 +387,19 @@ template <int KT, bool TWO>
 __device__ __forceinline__ void derivatives(const GroupView& g, const Lane<KT, TWO>& l, const NewV& nv, const bf* VV,
                                             bf* DG, const bf* EN, const int* cexp) {
     Out d;
-    const uint4* D1 = (const uint4*)g.D1MM;
     if (!TWO || l.eta) {
         if (TWO) l.sync();
-        product<KT, true>(D1, EN, l.S, l.w, d);
-        l.write(g, 4, d);
-    }
-    l.sync_both();
-    if (TWO && l.eta) {
-        product<KT, true>(D1, VV, l.S, l.w, d);
-        l.write(g, 1, d);
-        return;
+#pragma unroll 1
+        for (int f = 4; f > 0; f -= 3) {        // D eta, then D v
+            product<KT, true>((const uint4*)g.D1MM, f == 4 ? EN : VV, l.S, l.w, d);
+            l.write(g, f, d);
+            if (f == 4) l.sync_both();
+        }
+        if (TWO) return;
+    } else {
+        l.sync_both();
     }
     stage_digits(l.S, l.w, nv, DG, cexp);
-    if (!TWO) {
-        product<KT, true>(D1, VV, l.S, l.w, d);
-        l.write(g, 1, d);
-    }
     l.sync();
     d2_product<KT>(g, DG, l.S, l.w, d);
     l.write(g, 2, d);
@@ -578,8 +575,8 @@ struct Field {
                 const float2 m = s == 2 ? R.m1[r][k2] : dm.nat(r, l.pair[r], k2), pp = dp.nat(r, l.pair[r], k2);
                 const size_t h = l.h(r, k2);
                 if (s == 1) M1[h] = m;
-                R.x[r][k2].x += f2d(__fadd_rn(m.x, pp.x));
-                R.x[r][k2].y += f2d(__fadd_rn(m.y, pp.y));
+                R.x[r][k2].x += (double)__fadd_rn(m.x, pp.x);
+                R.x[r][k2].y += (double)__fadd_rn(m.y, pp.y);
                 O[h] = R.x[r][k2];
                 xs[r][k2] = make_float2(d2f(R.x[r][k2].x), d2f(R.x[r][k2].y));
                 P[l.o(r, k2)] = xs[r][k2];
@@ -629,26 +626,33 @@ __global__ void __maxnreg__(REGS) k_spec_mma(GroupView g, int s) {
         float2 nu[2][2], nw[2][2];
         fv.load(Rv, nu, nw);
         fe.load_acc(Re);
-        fe.load_x(Re);
-        if (fv.needM) fv.load_x(Rv);
+        if (fv.needM) {
+            fe.load_x(Re);
+            fv.load_x(Rv);
+        }
         fv.terms(Rv, nu, nw, xs);
         put_parts(VV, l.S, l.w, l.pair, xs);
         fe.terms(Re, nu, nw, xs);
         put_parts(GT, l.S, l.w, l.pair, xs);
         fe.put_x(Re, XE);
         fv.put_x(Rv, XV);
-        fe.load_m1(Re);
         l.sync();
         fv.forcing(Rv, VV, FT);
-        fe.increment(XE, dm);
-        fe.apply(Re, dm, GT, xs);
-        put_parts(EN, l.S, l.w, l.pair, xs);
-        fv.load_x(Rv);                          // again: not held across the eta phase
-        fv.load_m1(Rv);
-        l.sync();
-        fv.increment(XV, dm);
-        fv.apply(Rv, dm, FT, xs);
-        stage_v(l.S, l.w, l.pair, Rv.x, nv, VV, cexp);
+        // eta, then v: rolled, as is every other loop whose turns share their code (a
+        // warp runs the kernel once, top to bottom, and instruction fetch is what it
+        // waits for most)
+#pragma unroll 1
+        for (int eta = 1; eta >= 0; --eta) {
+            const Field<KT, TWO> f(g, l, s, eta != 0);
+            Rows R;
+            f.load_x(R);
+            f.load_m1(R);
+            if (!eta) l.sync();
+            f.increment(eta ? XE : XV, dm);
+            f.apply(R, dm, eta ? GT : FT, xs);
+            if (eta) put_parts(EN, l.S, l.w, l.pair, xs);
+            else stage_v(l.S, l.w, l.pair, R.x, nv, VV, cexp);
+        }
     }
     derivatives<KT, TWO>(g, l, nv, VV, GT, EN, cexp);
 }
