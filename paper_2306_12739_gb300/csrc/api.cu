@@ -1048,6 +1048,47 @@ static void drop_graphs(dns_handle* h) {
 
 static int new_state_derivatives(dns_handle* h, const GroupView& v, cudaStream_t st);
 
+// Milliseconds of a whole step of the handle as it is set up now, as dns_step will
+// run it: replays of a captured graph (an eager step of many small launches is
+// bound by the host, which hides what the candidates differ by: 64x65x64 x 8, the
+// fused against the step-by-step stage 308 and 305 us eager, 294 and 305 replayed),
+// or eager steps where the handle runs without graphs.
+static int time_step(dns_handle* h, float* ms) {
+    const int reps = h->cfg.use_graph && h->stream ? 8 : 3;
+    cudaStream_t st = h->stream;
+    cudaGraph_t gr = nullptr;
+    cudaGraphExec_t ex = nullptr;
+    int rc = DNS_OK;
+    if (h->cfg.use_graph && st) {
+        if ((rc = check(h, cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal), "begin capture"))) return rc;
+        enqueue_step(h);
+        rc = check(h, cudaStreamEndCapture(st, &gr), "end capture");
+        if (!rc) rc = check(h, cudaGraphInstantiate(&ex, gr, 0), "instantiate graph");
+    }
+    auto step = [&]() {
+        if (ex) cudaGraphLaunch(ex, st);
+        else enqueue_step(h);
+    };
+    cudaEvent_t e0, e1;
+    cudaEventCreate(&e0);
+    cudaEventCreate(&e1);
+    if (!rc) {
+        for (int w = 0; w < 2; ++w) step();
+        cudaEventRecord(e0, st);
+        for (int r = 0; r < reps; ++r) step();
+        cudaEventRecord(e1, st);
+        rc = check(h, cudaEventSynchronize(e1), "autotune whole step");
+        if (!rc) cudaEventElapsedTime(ms, e0, e1);
+        *ms /= (float)reps;
+    }
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    if (ex) cudaGraphExecDestroy(ex);
+    if (gr) cudaGraphDestroy(gr);
+    h->launches = 0;
+    return rc;
+}
+
 int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
     NvtxRange range_("dns_bind_workspace");
     if (!h) return DNS_ERR_INVALID;
@@ -1267,9 +1308,6 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
         float t_choice = 0.f, t_sbs = 0.f;
         if (!choice) {
             float best[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            cudaEvent_t e0, e1;
-            cudaEventCreate(&e0);
-            cudaEventCreate(&e1);
             for (int cand = 1; cand <= 8 && !rc; ++cand) {
                 if (cand == 3 || (cand == 2 && !dnsk::helm_tc_supported(v0)) ||
                     (cand == 4 && !dnsk::spec_supported(v0)) || (cand == 5 && !fuse_ok) || (cand == 6 && !par_ok) ||
@@ -1283,17 +1321,8 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
                     vb.spec_eoff = cand == 7 ? 1 : 0;
                     vb.step_eo = cand == 8 ? 1 : 0;
                 }
-                for (int w = 0; w < 2; ++w) enqueue_step(h);
-                cudaEventRecord(e0, st);
-                for (int r = 0; r < 3; ++r) enqueue_step(h);
-                cudaEventRecord(e1, st);
-                rc = check(h, cudaEventSynchronize(e1), "autotune per-wavenumber stage");
-                if (!rc) cudaEventElapsedTime(&best[cand], e0, e1);
-                best[cand] /= 3.f;
+                rc = time_step(h, &best[cand]);
             }
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            h->launches = 0;
             if (rc) return rc;
             if ((rc = device_status(h))) return rc;
             choice = 0;
@@ -1446,28 +1475,16 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
         if (std::find(cands.begin(), cands.end(), choice) == cands.end()) choice = 0;
         if (!choice) {
             std::vector<float> ms(cands.size(), 0.f);
-            cudaEvent_t e0, e1;
-            cudaEventCreate(&e0);
-            cudaEventCreate(&e1);
             for (size_t ci = 0; ci < cands.size() && !rc; ++ci) {
                 for (const auto& P : h->parts[gi]) h->groups[P.ig].v.spec_minb = cands[ci];
-                for (int w = 0; w < 2; ++w) enqueue_step(h);
-                cudaEventRecord(e0, st);
-                for (int r = 0; r < 3; ++r) enqueue_step(h);
-                cudaEventRecord(e1, st);
-                rc = check(h, cudaEventSynchronize(e1), "autotune fused-stage CTAs per SM");
-                if (!rc) cudaEventElapsedTime(&ms[ci], e0, e1);
+                rc = time_step(h, &ms[ci]);
             }
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            h->launches = 0;
             if (rc) return rc;
             if ((rc = device_status(h))) return rc;
             size_t best = 0;
             for (size_t ci = 1; ci < cands.size(); ++ci)
                 if (ms[ci] < ms[best]) best = ci;
             choice = cands[best];
-            for (auto& m : ms) m /= 3.f;
             cache_store_shape(h->cfg.autotune_cache, key, choice, cands, ms);
         }
         decided[key] = choice;

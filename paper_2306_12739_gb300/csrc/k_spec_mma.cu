@@ -51,7 +51,10 @@ using spc::EoRows;
 typedef unsigned short bf;
 
 constexpr int EC_MAX = 8;      // members per CTA (two modes: 16 complex columns)
-constexpr int YD_EC = 2;       // members per CTA of the y-derivatives (one column tile each)
+// members per CTA of the y-derivatives (one column tile each): one from three row
+// tiles up, whose CTAs are then 6 or 8 warps and three fit an SM
+__host__ __device__ constexpr int yd_ec(int kt) { return kt > 2 ? 1 : 2; }
+__host__ __device__ constexpr int yd_regs(int kt) { return kt == 3 ? 112 : 128; }
 constexpr int PIECES = 3;
 
 __host__ __device__ inline int tiles(int ny) { return ((ny + 1) / 2 + 15) / 16; }   // 16-row tiles of a parity block
@@ -334,7 +337,7 @@ struct Lane {
         rows(g, live);
     }
     // the y-derivatives' columns: a column tile is 4 consecutive modes of one member
-    __device__ __forceinline__ Lane(const GroupView& g, int q0, int e0) : S(shape_of(g.ny, YD_EC)), c() {
+    __device__ __forceinline__ Lane(const GroupView& g, int q0, int e0) : S(shape_of(g.ny, yd_ec(KT))), c() {
         place(g);
         q = q0 + (w.lane & 3);
         e = e0 + w.nt;
@@ -698,15 +701,15 @@ __global__ void __maxnreg__(128) k_mma_derivs(GroupView g) {
     if (l.tile) state_derivatives<KT>(g, l, g.v_t, g.e_t, sm);
 }
 
-// The y-derivatives of the step-by-step stage: 4 consecutive modes x YD_EC members a
+// The y-derivatives of the step-by-step stage: 4 consecutive modes x yd_ec members a
 // CTA, so that the per-plane fields are written in whole sectors; the grid's rows
 // beyond the members finish the previous sub-step's mean flow.
 template <int KT>
-__global__ void __maxnreg__(128) k_yderiv_mma(GroupView g, const double2* __restrict__ V, const double2* __restrict__ H,
+__global__ void __maxnreg__(yd_regs(KT)) k_yderiv_mma(GroupView g, const double2* __restrict__ V, const double2* __restrict__ H,
                                               int sprev) {
     extern __shared__ __align__(16) unsigned char sm[];
-    if (mean_finish_rows(g, sprev, (g.E + YD_EC - 1) / YD_EC, sm)) return;
-    const Lane<KT, true> l(g, 4 * blockIdx.x, YD_EC * blockIdx.y);
+    if (mean_finish_rows(g, sprev, (g.E + yd_ec(KT) - 1) / yd_ec(KT), sm)) return;
+    const Lane<KT, true> l(g, 4 * blockIdx.x, yd_ec(KT) * blockIdx.y);
     if (l.tile) state_derivatives<KT>(g, l, V, H, sm);
 }
 
@@ -841,10 +844,10 @@ void launch_mma_derivs(const GroupView& g, cudaStream_t st) {
 }
 
 void launch_yderiv_mma(const GroupView& g, const double2* v, const double2* e, cudaStream_t st, int sprev) {
-    const int kt = smm::tiles(g.ny), threads = 64 * kt * smm::YD_EC;
-    dim3 grid((g.nmodes + 3) / 4, (g.E + smm::YD_EC - 1) / smm::YD_EC);
+    const int kt = smm::tiles(g.ny), ec = smm::yd_ec(kt), threads = 64 * kt * ec;
+    dim3 grid((g.nmodes + 3) / 4, (g.E + ec - 1) / ec);
     grid.y += mean_finish_extra_rows(g, grid.x, sprev);
-    size_t sm = smm::smem_bytes(smm::shape_of(g.ny, smm::YD_EC), 4);
+    size_t sm = smm::smem_bytes(smm::shape_of(g.ny, ec), 4);
     if (sm < mean_smem_bytes(g)) sm = mean_smem_bytes(g);
 #define DNS_CASE(k) if (kt == k) smm::k_yderiv_mma<k><<<grid, threads, sm, st>>>(g, v, e, sprev);
     DNS_CASE(1) DNS_CASE(2) DNS_CASE(3) DNS_CASE(4)
