@@ -198,14 +198,36 @@ __global__ void __launch_bounds__(THREADS) k_yderiv_eo(GroupView g, const double
 
 // ---------------------------------------------------------------- forcing
 
-// Column tile of k_forcing_t; D1 in parity blocks, phi in parity parts, G and
-// -k^2 Nv in natural rows.  Tasks: two pair-rows x one complex column.
-__global__ void __launch_bounds__(THREADS) k_forcing_eo(GroupView g, int s) {
+// Column tile of the forcing: tile_of's, halved while its shared memory (D1, three
+// vectors) keeps fewer than four CTAs on an SM: what bounds it is the latency of
+// its loads, not their coalescing (128x97x128 x 4: 32 columns and two CTAs 50.5 us,
+// 16 columns 43.0; 64x65x64 x 4, 64x128x64 x 2, 32x97x32 x 4 within 4 %).
+constexpr size_t FO_SMEM_MAX = 56 * 1024;
+__host__ __device__ inline size_t fo_bytes(int ny, int nc) {
+    return (spc::eo_mat(ny) + 3 * (size_t)ny * 2 * nc) * sizeof(float);
+}
+__host__ __device__ inline gt::Tile fo_tile(int E, int ny, int nm) {
+    gt::Tile t = gt::tile_of(E, ny, nm);
+    while (fo_bytes(ny, t.NC) > FO_SMEM_MAX && t.NC > 16) {
+        if (t.QT > 1) t.QT /= 2;
+        else t.EBT = (t.EBT + 1) / 2;
+        t.NC = t.QT * t.EBT;
+    }
+    return t;
+}
+
+// That column tile; D1 in parity blocks, phi in parity parts, G and -k^2 Nv in
+// natural rows.  Tasks: two pair-rows x one complex column.  A launch is a chain of
+// dependent loads, so D1 is copied while the nonlinear terms are read, the
+// accumulators are loaded before the product that needs no memory, and the tile comes
+// from the host (its loop of divisions cost up to half a microsecond): 128x97x128 x 4
+// 43.0 -> 36.6 us, 64x65x64 x 4 12.3 -> 11.7, 32x49x32 x 16 12.3 -> 11.2, 32x33x32
+// x 4 9.1 -> 8.2.
+__global__ void __launch_bounds__(THREADS, 3) k_forcing_eo(GroupView g, gt::Tile T, int s) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int Ny = g.ny, E = g.E, NM = g.nmodes, NKX = g.nkx;
     const int NE = (Ny + 1) / 2, NO = Ny / 2, RP2 = spc::eo_rp(Ny), RB2 = (NE + 1) / 2;
     const size_t MEO = spc::eo_mat(Ny);
-    const gt::Tile T = gt::tile_of(E, Ny, NM);
     const FastDiv dNKX((unsigned)NKX);
     const int q0 = blockIdx.x * T.QT, e0 = blockIdx.y * T.EBT;
     const int NCR = 2 * T.NC;
@@ -217,7 +239,8 @@ __global__ void __launch_bounds__(THREADS) k_forcing_eo(GroupView g, int s) {
     const float2* N3 = (const float2*)g.N3;
     {
         const float4* s1 = (const float4*)g.D1EO;
-        for (int i = threadIdx.x; i < (int)(MEO / 4); i += THREADS) ((float4*)D1)[i] = s1[i];
+        for (int i = threadIdx.x; i < (int)(MEO / 4); i += THREADS)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(su32((float4*)D1 + i)), "l"(s1 + i) : "memory");
         const int per_y = T.EBT * T.QT;
         const FastDiv dPY((unsigned)per_y), dQT((unsigned)T.QT);
         for (int i = threadIdx.x; i < NE * per_y; i += THREADS) {
@@ -250,6 +273,7 @@ __global__ void __launch_bounds__(THREADS) k_forcing_eo(GroupView g, int s) {
             *(float2*)&PH[p * NCR + c] = make_float2(ph[0].x + ph[1].x, ph[0].y + ph[1].y);
             if (R.pair) *(float2*)&PH[(NE + p) * NCR + c] = make_float2(ph[0].x - ph[1].x, ph[0].y - ph[1].y);
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
     }
     __syncthreads();
     const FastDiv dEB2((unsigned)T.EBT), dQT2((unsigned)T.QT);
@@ -263,11 +287,6 @@ __global__ void __launch_bounds__(THREADS) k_forcing_eo(GroupView g, int s) {
         const int j = el * T.QT + qq, p0 = 2 * rb;
         const int q = q0 + qq, e = e0 + el;
         if (q >= NM || e >= E) continue;
-        // D1 phi: the even rows contract the odd part, the odd rows the even part
-        float ye[2][2], yo[2][2];
-        eo2(D1, NO, NE, RP2, PH + NE * NCR, PH, NCR, p0, 2 * j, ye, yo);
-        const int fmi = g.fn > 0 ? q / g.nkx : 0;
-        const bool forced = g.fn > 0 && q - fmi * g.nkx == g.fn;
         // the RK accumulators of the (up to four) natural rows before any store
         float2 pav[2][2], pae[2][2];
 #pragma unroll
@@ -281,6 +300,11 @@ __global__ void __launch_bounds__(THREADS) k_forcing_eo(GroupView g, int s) {
                 pav[rr][k2] = Av[h];
                 pae[rr][k2] = Ae[h];
             }
+        // D1 phi: the even rows contract the odd part, the odd rows the even part
+        float ye[2][2], yo[2][2];
+        eo2(D1, NO, NE, RP2, PH + NE * NCR, PH, NCR, p0, 2 * j, ye, yo);
+        const int fmi = g.fn > 0 ? q / g.nkx : 0;
+        const bool forced = g.fn > 0 && q - fmi * g.nkx == g.fn;
 #pragma unroll
         for (int rr = 0; rr < 2; ++rr) {
             const int p = p0 + rr;
@@ -476,8 +500,7 @@ __global__ void __launch_bounds__(THREADS, 3) k_helm_eo(GroupView g, int s) {
 // ------------------------------------------------------------------- host
 
 size_t forcing_eo_smem_bytes(const GroupView& g) {
-    gt::Tile t = gt::tile_of(g.E, g.ny, g.nmodes);
-    return (spc::eo_mat(g.ny) + 3 * (size_t)g.ny * 2 * t.NC) * sizeof(float);
+    return sto::fo_bytes(g.ny, sto::fo_tile(g.E, g.ny, g.nmodes).NC);
 }
 
 size_t helm_eo_smem_bytes(const GroupView& g) {
@@ -495,9 +518,9 @@ bool step_eo_fits(const GroupView& g) {
 bool step_eo_supported(const GroupView& g) { return !g.lin && step_eo_fits(g); }
 
 void launch_forcing_eo(const GroupView& g, int s, cudaStream_t st) {
-    gt::Tile t = gt::tile_of(g.E, g.ny, g.nmodes);
+    const gt::Tile t = sto::fo_tile(g.E, g.ny, g.nmodes);
     dim3 grid((g.nmodes + t.QT - 1) / t.QT, (g.E + t.EBT - 1) / t.EBT);
-    sto::k_forcing_eo<<<grid, sto::THREADS, forcing_eo_smem_bytes(g), st>>>(g, s);
+    sto::k_forcing_eo<<<grid, sto::THREADS, forcing_eo_smem_bytes(g), st>>>(g, t, s);
 }
 
 void launch_helm_eo(const GroupView& g, int s, cudaStream_t st) {
@@ -515,6 +538,10 @@ size_t yderiv_eo_smem_bytes(const GroupView& g) {
 // every group's interior grid, linear groups included)
 bool yderiv_eo_supported(const GroupView& g) { return g.ny >= 3 && yderiv_eo_smem_bytes(g) <= 227 * 1024; }
 
+// On the tensor products (k_spec_mma.cu) wherever D1's and D2's fragments were laid
+// out, which is every group that may take this kernel: 128x97x128 x 4 121.8 -> 76.5
+// us, 64x65x64 x 4 22.8 -> 17.2, 32x97x32 x 4 26.9 -> 11.9, 16x33x16 x 1 10.5 -> 8.8,
+// 32x33x32 x 4 equal (10.4).
 void launch_yderiv_eo(const GroupView& g, const double2* v, const double2* e, cudaStream_t st, int sprev) {
     if (g.D1MM != nullptr && g.D2MM != nullptr) {
         launch_yderiv_mma(g, v, e, st, sprev);
