@@ -255,6 +255,13 @@ def spec_computes_d2v(g):
     return g.get("_stage") in ("fused_d2v", "fused_eo_ff") or g["my"] - 2 > 64
 
 
+def runs_class(cls, g):
+    """The group's per-wavenumber stage launches this kernel class: the fused stages
+    "spec", the step-by-step ones "yderiv", "forcing" and "helm"."""
+    fused = str(g.get("_stage", "")).startswith("fused")
+    return fused if cls == "spec" else not fused if cls in ("yderiv", "forcing", "helm") else True
+
+
 def member_blocks(g):
     """Member blocks a group runs as (the library's rule: E/4 clamped to [4, 16],
     one block below 8 members, shared-mean and linear groups one block)."""
@@ -661,8 +668,8 @@ def gpu_arm(args, rank, world, dist):
     dom = max(kt, key=lambda k: kt[k][0])
     # every member of every group passes through the kernel once per sub-step
     # (member blocks split a group over several launches; the work is per member)
-    work = sum(kernel_work(dom, g, precision)[1] for g in groups) * 3 * n_timed
-    dbytes = sum(kernel_bytes(dom, g, precision) for g in groups) * 3 * n_timed
+    work = sum(kernel_work(dom, g, precision)[1] for g in groups if runs_class(dom, g)) * 3 * n_timed
+    dbytes = sum(kernel_bytes(dom, g, precision) for g in groups if runs_class(dom, g)) * 3 * n_timed
     avg_ms = kt[dom][0] / max(1, kt[dom][1])
     kprec = kernel_precision(dom, precision)
     sm_mhz = clocks["sm_mhz"] or 2070.0
@@ -686,7 +693,7 @@ def gpu_arm(args, rank, world, dist):
     # event pass runs the kernels one at a time)
     per_class = {}
     for cls, (ms, nl) in kt.items():
-        b = sum(kernel_bytes(cls, g, precision) for g in groups) * 3 * n_timed
+        b = sum(kernel_bytes(cls, g, precision) for g in groups if runs_class(cls, g)) * 3 * n_timed
         if b <= 0 or ms <= 0:
             continue
         gbs = b / (ms / 1e3) / 1e9

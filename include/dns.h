@@ -157,7 +157,7 @@ typedef struct {
     int helm;                      /* mixed path per-wavenumber stage: 0 autotuned at
                                       dns_bind_workspace (DNS groups: 1, 2 and 8, each timed with
                                       the y-derivatives and the forcing, against 4 to 7; linear
-                                      groups: 1 against 2),
+                                      groups: 1, 2 and 8, the last with the forcing),
                                       1 register-tiled FP32 implicit apply (one CTA per
                                       wavenumber pair and field), 2 tcgen05 tensor cores with
                                       split-BF16 operands (groups with My <= 66 and <= 64 members;
@@ -179,7 +179,11 @@ typedef struct {
                                       the operator bytes and multiply-adds (groups whose D2 v
                                       comes from the tensor-core kernel; others run 4), 7 the
                                       same with D2 v summed inside it in float-float (D2 in
-                                      parity blocks; every size the fused stage takes), 8 the
+                                      parity blocks; every size the fused stage takes; where
+                                      the group's operators as matrix fragments take at most
+                                      96 MB its products run on the warp-level tensor
+                                      instructions, three BF16 pieces per factor and D2 v as
+                                      exact digit products), 8 the
                                       step-by-step stage of 1 with its forcing (D1) and implicit
                                       apply (M - I, P) in parity blocks (DNS groups; linear
                                       groups and tiles that do not fit run 1) */
@@ -347,7 +351,7 @@ enum {
     DNS_K_FORCING = 3,     /* F, G and the RK3 combination */
     DNS_K_HELM = 4,        /* per-wavenumber implicit apply */
     DNS_K_MEAN = 5,        /* mean flow + constant-flux gamma */
-    DNS_K_SPEC = 6,        /* fused per-wavenumber stage (helm = 4): forcing, RK3 combination,
+    DNS_K_SPEC = 6,        /* fused per-wavenumber stage (helm = 4 to 7): forcing, RK3 combination,
                               implicit apply, y-derivatives of the new state, mean flow */
     DNS_K_D2V = 7,         /* D2 v of the new state on tensor cores (with the fused stage, My <= 66) */
     DNS_K_NCLASS = 8

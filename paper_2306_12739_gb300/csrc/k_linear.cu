@@ -58,8 +58,10 @@ using namespace prs;
 // lane does the residues 2 j and 2 j + 1 modulo N2 as a pair, then N2-point DFTs
 // whose two halves are the rows p and p + Mz/2), so only the products between the
 // inverse and the forward transforms need the CTA together.  61 planes x 45 vectors
-// of 64 points: 16.7 us a launch with a Stockham transform of the nine lines of one
-// vector per CTA, a barrier per radix-4 pass.
+// of 64 points: 16.6 us a launch alone with a Stockham transform of the nine lines of
+// one vector per CTA, a barrier per radix-4 pass, 18.5 here; but a launch takes less of
+// the chip, and groups run side by side: 3 x 45 vectors, 20 + 20 steps with
+// Gram-Schmidt 10270 -> 9790 us.
 template <int MZ> struct LinCfg {
     static constexpr int N1 = dft::Split<MZ>::N1, N2 = dft::Split<MZ>::N2, H = N2 / 2, HP = MZ / 2;
     static constexpr int NV = 32 / H;                         // vectors of a CTA
