@@ -145,8 +145,10 @@ typedef struct {
                                       against 1 and 3 only up to My = 49 (linear groups at every
                                       size); 1 and 3 are timed against each other at every size */
     int plane;                     /* plane stage: 0 autotuned where several kernels exist (else
-                                      the only one; 5 for FP64 and for 128-point grids where the
-                                      size has it), 1 one CTA per plane
+                                      the only one; 5, where the size has it, for FP64, for
+                                      128-point grids, and for mixed advective groups with Mx
+                                      and Mz of at least 32 and 1.5 million interior points
+                                      (My - 2) Mx Mz members or more), 1 one CTA per plane
                                       (sizes <= 64), 2 a thread-block cluster per plane (64x64
                                       single precision, and every size with a 128), 3 one CTA
                                       per plane with each 1-D transform owned by one group of

@@ -599,16 +599,18 @@ bool plane_variant_ok(bool mixed, const GroupView& v, int c) {
 // kernel is asked for:
 //   128-point grids, where a plane does not fit one SM: 404 -> 153 us a launch
 //   against the cluster kernel on 128x97x128 x 4, 1099 -> 670 us in FP64;
-//   FP64 everywhere: 991 -> 548 us on 64x65x64 x 4, 154 -> 144 on 32x33x32 x 2; the single-CTA kernel spends its FP64 pipe on
-//   radix-2 to 4 passes and leaves SMs idle at few planes;
-//   large mixed advective groups (1.5 M interior points over all members, both
+//   FP64 everywhere: 991 -> 548 us on 64x65x64 x 4, 154 -> 144 on 32x33x32 x 2; the
+//   single-CTA kernel spends its FP64 pipe on radix-2 to 4 passes and leaves SMs idle at
+//   few planes;
+//   large mixed advective groups (1.5 M interior points over all the group's members,
+//   not a block's, so that every block of a group runs the same kernel; both
 //   lengths 32 and more), whose launches fill the chip several times, so that the
 //   fewer instructions count and the two extra launches do not: whole steps of
 //   32x49x32 x 64 496 -> 411 us, x 32 271 -> 240, x 16 169 -> 177; 64x65x64 x 8
 //   331 -> 324, x 4 174 -> 187; in the rotational form (fewer transforms) 282 -> 298.
-bool plane_split_default(const GroupView& v, bool mixed) {
+bool plane_split_default(const GroupView& v, int members, bool mixed) {
     if (!mixed || v.mx == 128 || v.mz == 128) return true;
-    const double points = (double)v.ny * v.E * v.nblk * v.mx * v.mz;
+    const double points = (double)v.ny * members * v.mx * v.mz;
     return !v.rot && v.mx >= 32 && v.mz >= 32 && points >= 1.5e6;
 }
 
@@ -764,7 +766,7 @@ int choose_variants(dns_handle* h, const dns_config* cfg, GroupView& v, int gi) 
         v.plane = navail == 1 ? (ok[1] ? 1 : ok[2] ? 2 : 3) : (mixed ? 0 : 1);
         if (navail > 1 && cfg->plane >= 1 && cfg->plane <= 3 && ok[cfg->plane]) v.plane = cfg->plane;
         if (dnsk::plane_split_supported(v) && (cfg->plane == 5 || (!(cfg->plane >= 1 && cfg->plane <= 3 && ok[cfg->plane]) &&
-                                                                   plane_split_default(v, mixed))))
+                                                                   plane_split_default(v, d.members, mixed))))
             v.plane = 5;
     }
     if (precision_mixed(h)) {
