@@ -13,9 +13,13 @@
 // Precision: every single-precision factor is written as three BF16 pieces (24
 // significant bits) and the six products that reach 2^-24 of the leading one are
 // accumulated in single precision, smallest first.  D2 v, whose rows cancel
-// beyond single precision, is an exact digit product as in k_d2v_tc.cu (six
-// signed 7-bit digits of both factors, the six levels whose digit numbers sum to
-// at most 5, each summed exactly), in parity blocks.
+// beyond single precision, is a product of signed 8-bit digits in parity blocks: eight
+// (seven up to My = 34) of each factor, D2's against its row's largest entry, v's
+// against its column's, the levels of digit products down to the last digit's, summed
+// without error.  What that leaves out is below a float-float sum's error at every
+// size (smooth columns, relative to max |D2 v|: 2.6e-13 against 8.8e-13 at My = 33,
+// 7.5e-13 against 5.8e-12 at 65, 3.3e-12 against 1.2e-11 at 97, 7.6e-12 against 2.9e-11
+// at 129), so that the rounding to single precision, 5e-8, is all that shows.
 //
 // One CTA per (pair (n, |m|), member chunk).  A warp has 16 pair-rows x 4 complex
 // columns (8 real ones); a lane owns two pair-rows of one column (their even and
@@ -36,7 +40,7 @@
 #include "eo.cuh"
 #include "ff.cuh"
 #include "mean.cuh"
-#include "oz.cuh"
+#include "mbar.cuh"
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -56,6 +60,11 @@ constexpr int EC_MAX = 8;      // members per CTA (two modes: 16 complex columns
 __host__ __device__ constexpr int yd_ec(int kt) { return kt > 2 ? 1 : 2; }
 __host__ __device__ constexpr int yd_regs(int kt) { return kt == 3 ? 112 : 128; }
 constexpr int PIECES = 3;
+// D2 v: signed digits of DBITS bits of either factor (at most 256 units, exact in
+// BF16); the levels s + t < ndig of the digit products are summed.  Seven digits leave
+// less than a float-float sum up to My = 34 (one row tile), eight at every size.
+constexpr int DBITS = 8;
+__host__ __device__ constexpr int ndig(int kt) { return kt == 1 ? 7 : 8; }
 
 __host__ __device__ inline int tiles(int ny) { return ((ny + 1) / 2 + 15) / 16; }   // 16-row tiles of a parity block
 // members per CTA: at most 512 threads
@@ -69,8 +78,12 @@ __host__ __device__ inline int col_tiles(int ec) { return (2 * ec + 3) / 4; }   
 // fragments: [block][row tile][k tile][piece or digit][lane] of 16 bytes
 __host__ __device__ constexpr int mat_frags(int kt, int n) { return 2 * kt * kt * n * 32; }
 
-// shared memory: 6 vectors of three pieces (phi / v+, G~, x_v, x_eta, F~, eta+; G~ and
-// x_eta then hold the six digits of v+), column exponents
+// shared memory: the stage 6 vectors of three pieces (phi / v+, G~, x_eta, x_v, F~, eta+;
+// the digits of v+ then lie over G~, x_eta and x_v), the derivatives alone v, its
+// digits and eta; column exponents
+constexpr int STAGE_PIECES = 6 * PIECES;
+__host__ __device__ constexpr int deriv_pieces(int kt) { return 2 * PIECES + ndig(kt); }
+static_assert(ndig(4) <= 3 * PIECES, "the digits lie over three vectors");
 struct Shape {
     int KT, NT, CS, VP;     // k tiles, column tiles, column stride and piece size (BF16 values)
 };
@@ -83,8 +96,8 @@ __host__ __device__ inline Shape shape_of(int ny, int nt) {
     return s;
 }
 __host__ __device__ inline Shape shape_of(const GroupView& g) { return shape_of(g.ny, col_tiles(chunk_members(g))); }
-inline size_t smem_bytes(const Shape& s, int vectors) {
-    return (size_t)vectors * PIECES * s.VP * sizeof(bf) + (size_t)s.KT * 8 * s.NT * sizeof(int);
+inline size_t smem_bytes(const Shape& s, int pieces) {
+    return (size_t)pieces * s.VP * sizeof(bf) + (size_t)s.KT * 8 * s.NT * sizeof(int);
 }
 
 __device__ __forceinline__ void mma(float (&d)[4], uint4 a, unsigned b0, unsigned b1) {
@@ -211,47 +224,54 @@ __device__ __forceinline__ void product(const uint4* __restrict__ A, const bf* v
     }
 }
 
+// h + b, the rounding error added to l
 __device__ __forceinline__ void two_sum(float& h, float& l, float b) {
     const float s = __fadd_rn(h, b), v = __fsub_rn(s, h);
     l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, v)), __fsub_rn(b, v)));
     h = s;
 }
-// D2 v: digit products level by level (a level's terms are multiples of one power
-// of two and sum exactly), the levels in float-float
+// D2 v: digit products level by level.  A level's terms are multiples of one power of
+// two and stay below 2^24 of it (64 columns, at most 8 products of a first digit up to
+// 256 or others up to 130), so each level sums exactly; the levels add up by error-free
+// transformations.  The last two levels share an accumulator: they weigh less than
+// 2^-40 of the scale, and cutting that off at 24 bits stays below what is left out.
+// up: the columns' powers of two.
 template <int KT>
-__device__ __forceinline__ void d2_product(const GroupView& g, const bf* dig, const Shape& S, const Place& w, Out& out) {
+__device__ __forceinline__ void d2_product(const GroupView& g, const bf* dig, const Shape& S, const Place& w, float2 up,
+                                           Out& out) {
+    constexpr int NDIG = ndig(KT), NACC = NDIG - 1;
     const unsigned at = su32(dig + (8 * w.nt + (w.lane & 7)) * S.CS + ((w.lane >> 3) & 1) * 8 + (w.lane >> 4) * S.VP);
 #pragma unroll 1
     for (int blk = 0; blk < 2; ++blk) {
-        const uint4* A = (const uint4*)g.D2MM + (size_t)blk * KT * KT * oz::NDIG * 32;
-        float acc[oz::NLEV][4];
+        const uint4* A = (const uint4*)g.D2MM + (size_t)blk * KT * KT * NDIG * 32;
+        float acc[NACC][4];
 #pragma unroll
-        for (int L = 0; L < oz::NLEV; ++L)
+        for (int L = 0; L < NACC; ++L)
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[L][i] = 0.f;
 #pragma unroll
         for (int kt = 0; kt < KT; ++kt) {
-            uint4 a[oz::NDIG];
+            uint4 a[NDIG];
 #pragma unroll
-            for (int s = 0; s < oz::NDIG; ++s) a[s] = A[((w.mt * KT + kt) * oz::NDIG + s) * 32 + w.lane];
+            for (int s = 0; s < NDIG; ++s) a[s] = A[((w.mt * KT + kt) * NDIG + s) * 32 + w.lane];
 #pragma unroll
-            for (int s = 0; s < oz::NDIG; s += 2) {
-                unsigned b[4];           // digits s, s + 1
+            for (int s = 0; s < NDIG; s += 2) {
+                unsigned b[4];           // digits s, s + 1 (beyond the last: whatever follows it, unused)
                 ldm4(b, at + 2 * (s * S.VP + 16 * KT * blk + 16 * kt));
 #pragma unroll
-                for (int L = s; L < oz::NLEV; ++L) mma(acc[L], a[L - s], b[0], b[1]);
+                for (int L = s; L < NDIG; ++L) mma(acc[L < NACC ? L : NACC - 1], a[L - s], b[0], b[1]);
 #pragma unroll
-                for (int L = s + 1; L < oz::NLEV; ++L) mma(acc[L], a[L - s - 1], b[2], b[3]);
+                for (int L = s + 1; L < NDIG; ++L) mma(acc[L < NACC ? L : NACC - 1], a[L - s - 1], b[2], b[3]);
             }
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            // levels 3 to 5 weigh less than 2^-18 of the scale: one sum
-            float h = acc[0][i], l = __fadd_rn(__fadd_rn(acc[5][i], acc[4][i]), acc[3][i]);
-            two_sum(h, l, acc[1][i]);
-            two_sum(h, l, acc[2][i]);
-            if (!blk) out.e[i] = __fadd_rn(h, l);
-            else out.o[i] = __fadd_rn(h, l);
+            float h = acc[0][i], l = 0.f;
+#pragma unroll
+            for (int L = 1; L < NACC - 1; ++L) two_sum(h, l, acc[L][i]);
+            const float r = __fmul_rn(__fadd_rn(h, __fadd_rn(l, acc[NACC - 1][i])), i & 1 ? up.y : up.x);
+            if (!blk) out.e[i] = r;
+            else out.o[i] = r;
         }
     }
 }
@@ -286,36 +306,49 @@ __device__ __forceinline__ void stage_v(const Shape& S, const Place& w, const bo
         if (w.lane < 4) cexp[w.mt * 8 * S.NT + 2 * w.j + c] = mx[c];
     }
 }
-// After a barrier: the digits of v's parts.  Digit s of x, |x| < 2^f, is the
-// multiple of 2^(f - 7 (s + 1)) nearest to what the digits before it leave (adding
-// and subtracting 1.5 2^23 units rounds to whole units): at most 2^7 units, exact
-// in BF16.  Beyond the third digit the float-float pair's low part joins in.
-__device__ __forceinline__ void stage_digits(const Shape& S, const Place& w, const NewV& nv, bf* DG, const int* cexp) {
+// After a barrier: the digits of v's parts, the column scaled by a power of two to
+// below 1 (a column of any magnitude keeps all of them); the result is that power.
+// Digit s is the multiple of 2^(-DBITS (s + 1)) nearest to what the digits before it
+// leave (adding and subtracting 1.5 2^23 units rounds to whole units).  The pair's low
+// part, below 2^-23, joins after the second digit as an error-free sum, whose error
+// joins after the fourth.
+template <int KT>
+__device__ __forceinline__ float2 stage_digits(const Shape& S, const Place& w, const NewV& nv, bf* DG, const int* cexp) {
+    float up[2];
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
         int be = 0;
         for (int m = 0; m < S.KT; ++m) be = max(be, cexp[m * 8 * S.NT + 2 * w.j + c]);
-        // 1.5 2^(f - 7 + 23), f = be - 126; columns below 2^-84 keep fewer digits
-        be = max(be, 43);
-        const unsigned magic0 = ((unsigned)min(be + 1 + 16, 254) << 23) | 0x400000u;
+        be = min(be, 252);                       // (beyond it, and for Inf and NaN, D2 v overflows)
+        up[c] = __uint_as_float((unsigned)(be + 1) << 23);                  // 2^f, f = be - 126
+        const float down = __uint_as_float((unsigned)(253 - be) << 23);     // 2^-f
         unsigned* o = (unsigned*)(DG + (2 * w.j + c) * S.CS + 16 * w.mt) + (w.lane >> 2);
 #pragma unroll
         for (int part = 0; part < 2; ++part) {
-            float r0 = part ? nv.oh[0][c] : nv.eh[0][c], r1 = part ? nv.oh[1][c] : nv.eh[1][c];
+            float r0 = __fmul_rn(part ? nv.oh[0][c] : nv.eh[0][c], down), l0 = __fmul_rn(part ? nv.ol[0][c] : nv.el[0][c], down);
+            float r1 = __fmul_rn(part ? nv.oh[1][c] : nv.eh[1][c], down), l1 = __fmul_rn(part ? nv.ol[1][c] : nv.el[1][c], down);
 #pragma unroll
-            for (int s = 0; s < oz::NDIG; ++s) {
-                const float m = __uint_as_float(magic0 - (unsigned)s * (7u << 23));
+            for (int s = 0; s < ndig(KT); ++s) {
+                const float m = __uint_as_float(((unsigned)(127 + 23 - DBITS * (s + 1)) << 23) | 0x400000u);
                 const float d0 = __fsub_rn(__fadd_rn(r0, m), m), d1 = __fsub_rn(__fadd_rn(r1, m), m);
                 o[s * (S.VP / 2) + 8 * S.KT * part] = __byte_perm(__float_as_uint(d0), __float_as_uint(d1), 0x7632);
                 r0 = __fsub_rn(r0, d0);
                 r1 = __fsub_rn(r1, d1);
-                if (s == 2) {
-                    r0 = __fadd_rn(r0, part ? nv.ol[0][c] : nv.el[0][c]);
-                    r1 = __fadd_rn(r1, part ? nv.ol[1][c] : nv.el[1][c]);
+                if (s == 1) {
+                    float e0 = 0.f, e1 = 0.f;
+                    two_sum(r0, e0, l0);
+                    two_sum(r1, e1, l1);
+                    l0 = e0;
+                    l1 = e1;
+                }
+                if (s == 3) {
+                    r0 = __fadd_rn(r0, l0);
+                    r1 = __fadd_rn(r1, l1);
                 }
             }
         }
     }
+    return make_float2(up[0], up[1]);
 }
 
 // A CTA's view of its work: the lane's column and natural rows
@@ -402,9 +435,9 @@ __device__ __forceinline__ void derivatives(const GroupView& g, const Lane<KT, T
     } else {
         l.sync_both();
     }
-    stage_digits(l.S, l.w, nv, DG, cexp);
+    const float2 up = stage_digits<KT>(l.S, l.w, nv, DG, cexp);
     l.sync();
-    d2_product<KT>(g, DG, l.S, l.w, d);
+    d2_product<KT>(g, DG, l.S, l.w, up, d);
     l.write(g, 2, d);
 }
 
@@ -599,8 +632,8 @@ __global__ void __maxnreg__(REGS) k_spec_mma(GroupView g, int s) {
     if (!l.tile) return;                        // only the warps of a column tile meet
     const int V = PIECES * l.S.VP;
     bf* VV = (bf*)sm;                           // phi, then v+
-    bf* GT = VV + V;                            // G~, then digits 0..2 of v+
-    bf* XE = GT + V;                            // eta_t, then digits 3..5
+    bf* GT = VV + V;                            // G~; the digits of v+ start here
+    bf* XE = GT + V;                            // eta_t
     bf* XV = XE + V;                            // v_t
     bf* FT = XV + V;                            // F~
     bf* EN = FT + V;                            // eta+
@@ -667,7 +700,7 @@ __device__ __forceinline__ void state_derivatives(const GroupView& g, const Lane
                                                   const double2* __restrict__ H, unsigned char* sm) {
     bf* VV = (bf*)sm;
     bf* DG = VV + PIECES * l.S.VP;
-    bf* EN = DG + 2 * PIECES * l.S.VP;
+    bf* EN = DG + ndig(KT) * l.S.VP;
     int* cexp = (int*)(EN + PIECES * l.S.VP);
     const double2* X = l.eta ? H : V;
     float2* P = (float2*)g.P5 + (l.eta ? 3 : 0) * l.fs5;
@@ -756,7 +789,7 @@ static void fragments(const double* eo, int ny, bool anti, int npiece, uint16_t*
 }
 
 size_t spec_mma_mat_bytes(int ny) { return (size_t)smm::mat_frags(smm::tiles(ny), smm::PIECES) * 16; }
-size_t spec_mma_d2_bytes(int ny) { return (size_t)smm::mat_frags(smm::tiles(ny), oz::NDIG) * 16; }
+size_t spec_mma_d2_bytes(int ny) { return (size_t)smm::mat_frags(smm::tiles(ny), smm::ndig(smm::tiles(ny))) * 16; }
 
 void spec_mma_image(const double* eo, int ny, bool anti, uint16_t* out) {
     fragments(eo, ny, anti, smm::PIECES, out, [](double v, int, int, int i) {
@@ -770,7 +803,7 @@ void spec_mma_image(const double* eo, int ny, bool anti, uint16_t* out) {
 }
 
 // D2's digits: digit i of a parity row whose entries are below 2^e is the multiple
-// of 2^(e - 7 (i + 1)) nearest to what the digits before it leave
+// of 2^(e - DBITS (i + 1)) nearest to what the digits before it leave
 void spec_mma_d2_image(const double* eo, int ny, uint16_t* out) {
     const int KT = smm::tiles(ny), NE = spc::eo_ne(ny), NO = ny / 2, RP = spc::eo_rp(ny);
     std::vector<int> rexp(2 * 16 * KT, 0);
@@ -781,11 +814,11 @@ void spec_mma_d2_image(const double* eo, int ny, uint16_t* out) {
             for (int k = 0; k < (blk ? NO : NE); ++k) mx = std::fmax(mx, std::fabs(B[(size_t)k * RP + r]));
             if (mx > 0.0) std::frexp(mx, &rexp[blk * 16 * KT + r]);
         }
-    fragments(eo, ny, false, oz::NDIG, out, [&](double v, int blk, int r, int i) {
+    fragments(eo, ny, false, smm::ndig(KT), out, [&](double v, int blk, int r, int i) {
         double d = 0.0;
         for (int s = 0; s <= i; ++s) {
             v -= d;
-            const double u = std::ldexp(1.0, rexp[blk * 16 * KT + r] - 7 * (s + 1));
+            const double u = std::ldexp(1.0, rexp[blk * 16 * KT + r] - smm::DBITS * (s + 1));
             d = std::nearbyint(v / u) * u;
         }
         return bf16_of(d);
@@ -797,12 +830,12 @@ void spec_mma_d2_image(const double* eo, int ny, uint16_t* out) {
 // L2, or streaming them costs more than the products save (128x97x128: 206 MB a
 // step length).
 bool spec_mma_supported(const GroupView& g) {
-    return !g.lin && g.npairs > 1 && g.ny >= 3 && smm::smem_bytes(smm::shape_of(g), 6) + 1024 <= 227 * 1024 &&
+    return !g.lin && g.npairs > 1 && g.ny >= 3 && smm::smem_bytes(smm::shape_of(g), smm::STAGE_PIECES) + 1024 <= 227 * 1024 &&
            2 * (size_t)g.npairs * 4 * spec_mma_mat_bytes(g.ny) <= ((size_t)96 << 20);
 }
 
 size_t spec_mma_smem_bytes(const GroupView& g) {
-    const size_t b = smm::smem_bytes(smm::shape_of(g), 6), m = mean_smem_bytes(g);
+    const size_t b = smm::smem_bytes(smm::shape_of(g), smm::STAGE_PIECES), m = mean_smem_bytes(g);
     return b > m ? b : m;
 }
 
@@ -847,7 +880,7 @@ void launch_yderiv_mma(const GroupView& g, const double2* v, const double2* e, c
     const int kt = smm::tiles(g.ny), ec = smm::yd_ec(kt), threads = 64 * kt * ec;
     dim3 grid((g.nmodes + 3) / 4, (g.E + ec - 1) / ec);
     grid.y += mean_finish_extra_rows(g, grid.x, sprev);
-    size_t sm = smm::smem_bytes(smm::shape_of(g.ny, ec), 4);
+    size_t sm = smm::smem_bytes(smm::shape_of(g.ny, ec), smm::deriv_pieces(kt));
     if (sm < mean_smem_bytes(g)) sm = mean_smem_bytes(g);
 #define DNS_CASE(k) if (kt == k) smm::k_yderiv_mma<k><<<grid, threads, sm, st>>>(g, v, e, sprev);
     DNS_CASE(1) DNS_CASE(2) DNS_CASE(3) DNS_CASE(4)
