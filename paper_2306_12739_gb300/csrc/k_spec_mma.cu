@@ -178,17 +178,31 @@ struct Out {
     }
 };
 
+// The tensor cores cut a sum off towards zero.  What that takes on average, in units in
+// the last place (emulated on the sums of this library's operators, My = 33 to 97, smooth
+// and rough columns; the instruction itself was seen to do it on random sums): of the
+// products of P 0.2 to 0.5, whose terms spread over many powers of two, of M - I 0.06 to
+// 0.36, of D1 0.02 to 0.27, mostly below 0.1 (many of its sums need no cut).  Left alone
+// it makes every increment a little too small, step after step: against 64 bits, after
+// 20 to 50 steps, errors of the state up to 1.18 times the FP32 stage's (32x24x32
+// rotational; 64x28x16 1.11, 48x36x32 1.04).  So P's leading sums get half a unit back
+// (to the small products' accumulator), M - I's a quarter: 0.90, 0.88 and 0.89 times.
+constexpr float CUT_P = 0x1p-24f, CUT_M = 0x1p-25f;     // of the sum's power of two
+
+// the power of two of x's binary exponent, x's sign
+__device__ __forceinline__ float power_of(float x) { return __uint_as_float(__float_as_uint(x) & 0xFF800000u); }
+
 // out = matrix x vector for this warp's tile.  SWAP: an anti-centro-symmetric
-// matrix (D1): its even rows contract the odd part, its odd rows the even part.
+// matrix (D1): its even rows contract the odd part, its odd rows the even part; its sums
+// are left as they are, those of the others get cut.
 template <int KT, bool SWAP>
 __device__ __forceinline__ void product(const uint4* __restrict__ A, const bf* vec, const Shape& S, const Place& w,
-                                        Out& out) {
+                                        Out& out, float cut = 0.f) {
     // this lane's row address of the four 8 x 8 blocks of an ldmatrix: columns of
     // the tile, k halves, parts
     const unsigned at = su32(vec + (8 * w.nt + (w.lane & 7)) * S.CS + ((w.lane >> 3) & 1) * 8 + (w.lane >> 4) * 16 * KT);
-    // The tensor cores cut an accumulator off towards zero: the leading products of
-    // a k tile start from zero and are added up rounded to nearest, the small ones
-    // have an accumulator of their own.
+    // The leading products of a k tile start from zero and are added up rounded to
+    // nearest, the small ones have an accumulator of their own.
     float le[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int kt = 0; kt < KT; ++kt) {
@@ -215,6 +229,10 @@ __device__ __forceinline__ void product(const uint4* __restrict__ A, const bf* v
         for (int i = 0; i < 4; ++i) {
             out.e[i] = kt == 0 ? he[i] : __fadd_rn(out.e[i], he[i]);
             out.o[i] = kt == 0 ? ho[i] : __fadd_rn(out.o[i], ho[i]);
+            if (!SWAP) {
+                le[i] = __fmaf_rn(power_of(he[i]), cut, le[i]);
+                lo[i] = __fmaf_rn(power_of(ho[i]), cut, lo[i]);
+            }
         }
     }
 #pragma unroll
@@ -594,13 +612,13 @@ struct Field {
         put_parts(FT, l.S, l.w, l.pair, t);
     }
     __device__ __forceinline__ void increment(const bf* XT, Out& dm) const {
-        if (needM) product<KT, false>(ops, XT, l.S, l.w, dm);
+        if (needM) product<KT, false>(ops, XT, l.S, l.w, dm, CUT_M);
     }
     // x+ = x_t + ((M - I) x_t + P F~): into the state, the per-plane field and R.x; its
     // single-precision rows in xs
     __device__ __forceinline__ void apply(Rows& R, const Out& dm, const bf* F, float2 (&xs)[2][2]) const {
         Out dp;
-        product<KT, false>(ops + mat_frags(KT, PIECES), F, l.S, l.w, dp);
+        product<KT, false>(ops + mat_frags(KT, PIECES), F, l.S, l.w, dp, CUT_P);
         float2* P = (float2*)g.P5 + (eta ? 3 : 0) * l.fs5;
 #pragma unroll
         for (int r = 0; r < 2; ++r)
