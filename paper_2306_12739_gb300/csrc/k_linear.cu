@@ -337,14 +337,15 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs_gather(GroupView g) {
     }
 }
 
-// Sum of the threads' values over the cluster, in a fixed order, times f; the
-// result in every thread.  On the FP64 pipe an addition costs a warp 16 cycles
-// of its SM, so one warp adds up the CTA and one thread the cluster.
+// Sum of the threads' values over the cluster, in a fixed order, divided by d; the
+// result in every thread.  inv is 1 / d, infinite for a subnormal d (vectors of norms
+// below 1e-154), which then divides.  On the FP64 pipe an addition costs a warp 16
+// cycles of its SM, so one warp adds up the CTA and one thread the cluster.
 struct GsShared {
     double2 lane[GS_THREADS];
     double2 part, sum;
 };
-__device__ __forceinline__ double2 cluster_sum(double2 v, double f, GsShared& sh) {
+__device__ __forceinline__ double2 cluster_sum(double2 v, double inv, double d, GsShared& sh) {
     cg::cluster_group cl = cg::this_cluster();
     sh.lane[threadIdx.x] = v;
     __syncthreads();
@@ -371,7 +372,7 @@ __device__ __forceinline__ double2 cluster_sum(double2 v, double f, GsShared& sh
             t.x += u.x;
             t.y += u.y;
         }
-        sh.sum = make_double2(t.x * f, t.y * f);
+        sh.sum = isinf(inv) ? make_double2(t.x / d, t.y / d) : make_double2(t.x * inv, t.y * inv);
     }
     cl.sync();       // the sum is there, and no peer reads this CTA's part any more
     return sh.sum;
@@ -420,7 +421,7 @@ __global__ void __cluster_dims__(GS_CL, 1, 1) __launch_bounds__(GS_THREADS, 3) k
             load(i, a, b);
             dot(a, b);
         }
-        c = cluster_sum(s, gs_inv(g)[k], sh);
+        c = cluster_sum(s, gs_inv(g)[k], gs_sq(g)[k], sh);
     }
     const bool norm = j == k + 1;
     double2 s = make_double2(0.0, 0.0);
@@ -444,7 +445,7 @@ __global__ void __cluster_dims__(GS_CL, 1, 1) __launch_bounds__(GS_THREADS, 3) k
     }
     if (norm) {
         __syncthreads();
-        s = cluster_sum(s, 1.0, sh);
+        s = cluster_sum(s, 1.0, 1.0, sh);
         if (rank == 0 && threadIdx.x == 0) {
             gs_sq(g)[j] = s.x;
             gs_inv(g)[j] = 1.0 / s.x;
