@@ -1053,21 +1053,28 @@ static int new_state_derivatives(dns_handle* h, const GroupView& v, cudaStream_t
 // Milliseconds of one call of run(): the shortest of three windows of n calls (in one
 // window a hiccup of a few tens of microseconds outweighs what candidates differ by:
 // 32x49x32 x 64 and 16x33x16 x 1 then ran 7 % and 4 % slower after one bind in two).
+// Calls that take long need fewer of them: n shrinks until a window is about 2 ms, by
+// a timed warm-up call (creating and binding the three-group batch, steps of 2.2 ms:
+// 3.4 -> 1.3 s, 128x97x128 x 16 6.95 -> 6.05, 32x49x32 x 64 0.26 -> 0.17; windows of 8 ms
+// choose the same).
 static int time_calls(dns_handle* h, cudaStream_t st, int n, const std::function<void()>& run, const char* what,
                       float* ms) {
+    constexpr float WINDOW_MS = 2.f;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     int rc = DNS_OK;
-    for (int w = 0; w < 2; ++w) run();
-    for (int w = 0; w < 3 && !rc; ++w) {
+    run();
+    for (int w = -1; w < 3 && !rc; ++w) {      // w = -1: the second warm-up call
+        const int calls = w < 0 ? 1 : n;
         float t = 0.f;
         cudaEventRecord(e0, st);
-        for (int r = 0; r < n; ++r) run();
+        for (int r = 0; r < calls; ++r) run();
         cudaEventRecord(e1, st);
         if ((rc = check(h, cudaEventSynchronize(e1), what))) break;
         cudaEventElapsedTime(&t, e0, e1);
-        if (w == 0 || t / (float)n < *ms) *ms = t / (float)n;
+        if (w < 0) n = std::max(1, std::min(n, (int)(WINDOW_MS / std::max(t, 1e-3f))));
+        else if (w == 0 || t / (float)n < *ms) *ms = t / (float)n;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
