@@ -1527,23 +1527,14 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
     // state (every block's, back to back), timed here on the workspace's contents
     for (size_t gi = 0; gi < h->parts.size() && !rc; ++gi) {
         if (!h->groups[h->parts[gi][0].ig].has_sbs) continue;
-        cudaEvent_t e0, e1;
-        cudaEventCreate(&e0);
-        cudaEventCreate(&e1);
         auto derivs = [&]() {
             for (const auto& P : h->parts[gi])
                 if (!rc) rc = new_state_derivatives(h, h->groups[P.ig].v, st);
         };
-        derivs();
-        cudaEventRecord(e0, st);
-        for (int r = 0; r < 3; ++r) derivs();
-        cudaEventRecord(e1, st);
         float ms = 0.f;
-        if (!rc) rc = check(h, cudaEventSynchronize(e1), "time the derivatives of a new state");
-        if (!rc) cudaEventElapsedTime(&ms, e0, e1);
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        for (const auto& P : h->parts[gi]) h->groups[P.ig].t_derivs = ms / 3.f;
+        const int rct = time_calls(h, st, 5, derivs, "time the derivatives of a new state", &ms);
+        if (!rc) rc = rct;
+        for (const auto& P : h->parts[gi]) h->groups[P.ig].t_derivs = ms;
     }
     h->launches = 0;
     if (rc) return rc;
