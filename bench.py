@@ -249,7 +249,7 @@ def kernel_work(cls, g, precision):
 
 def spec_computes_d2v(g):
     """The fused stage writes D2 v itself: with the digit product inside it
-    (per-wavenumber stage "fused_d2v"), in float-float (stage "fused_eo_ff", and
+    (per-wavenumber stage "fused_d2v"), in parity blocks (stage "fused_eo_ff", and
     above Ny = 64); else
     the separate tensor-core D2 v kernel does."""
     return g.get("_stage") in ("fused_d2v", "fused_eo_ff") or g["my"] - 2 > 64

@@ -137,9 +137,12 @@ typedef struct {
                                       register-tiled FP32 with D2 v summed in float-float, 2
                                       tcgen05 tensor cores with split-BF16 operands and FP32
                                       accumulation (groups with My <= 66 and <= 64 members), 3
-                                      the register-tiled kernel of 1 in parity blocks (D1 and
-                                      D2 as their even and odd halves; the same float-float
-                                      D2 v).  The FP32 accumulation of 2 loses about 1e-5 of
+                                      in parity blocks (D1 and D2 as their even and odd halves)
+                                      on the warp-level tensor instructions: three BF16 pieces
+                                      per factor, D2 v as products of signed 8-bit digits whose
+                                      error is below that of the float-float sum, so that both
+                                      round to the same accuracy.  The FP32 accumulation of 2
+                                      loses about 1e-5 of
                                       |D2 v| to the cancellation in D2's rows at My = 65, over
                                       the 1e-6 budget of the mixed step, so DNS groups time it
                                       against 1 and 3 only up to My = 49 (linear groups at every
@@ -169,8 +172,10 @@ typedef struct {
                                       starves concurrent member blocks), 4 the fused stage: one
                                       launch per sub-step does the forcing, RK3 combination,
                                       implicit apply, the y-derivatives of the new state and the
-                                      mean flow (DNS groups whose operators fit in shared memory:
-                                      My <= 99; linear groups use 1 or 2), 5 the fused stage
+                                      mean flow (DNS groups whose operators and columns fit in
+                                      shared memory: My <= 106 with one member in a member block,
+                                      98 with four, 89 with eight or more; linear groups are
+                                      autotuned among 1, 2 and 8), 5 the fused stage
                                       with D2 v of the new state computed inside the same launch
                                       (the tensor-core digit product of the separate D2 v
                                       kernel, bit for bit the same result; groups with
@@ -180,15 +185,15 @@ typedef struct {
                                       symmetric grid) applied as its even and odd halves, half
                                       the operator bytes and multiply-adds (groups whose D2 v
                                       comes from the tensor-core kernel; others run 4), 7 the
-                                      same with D2 v summed inside it in float-float (D2 in
-                                      parity blocks; every size the fused stage takes; where
-                                      the group's operators as matrix fragments take at most
-                                      96 MB its products run on the warp-level tensor
-                                      instructions, three BF16 pieces per factor and D2 v as
-                                      exact digit products), 8 the
+                                      same with D2 v inside it, in parity blocks (every size
+                                      the fused stage takes): where the group's operators as
+                                      matrix fragments take at most 96 MB, every product on the
+                                      warp-level tensor instructions as in ygemm 3, elsewhere
+                                      FP32 products and D2 v summed in float-float, 8 the
                                       step-by-step stage of 1 with its forcing (D1) and implicit
-                                      apply (M - I, P) in parity blocks (DNS groups; linear
-                                      groups and tiles that do not fit run 1) */
+                                      apply (M - I, P) in parity blocks (by request in DNS
+                                      groups only: a request for a linear group, or for tiles
+                                      that do not fit, runs 1) */
 } dns_config;
 
 /* One-point statistics of one member (paper Sec. 4), computed from the current
@@ -332,13 +337,14 @@ const char* dns_last_error(const dns_handle* h);
 
 /* Kernel variants `group` uses, after the autotuner ran (i.e. after
  * dns_bind_workspace): ygemm 1 register-tiled FP32 / 2 tcgen05 y-contraction /
- * 3 register-tiled FP32 in parity blocks;
+ * 3 in parity blocks on the warp-level tensor instructions;
  * plane 1 one CTA per plane / 2 a thread-block cluster per plane / 3 line-owned
  * single CTA per plane / 5 three launches per plane stage (4 the linear groups'
  * own); helm 1 register-tiled FP32 / 2 tcgen05 implicit apply /
  * 3 persistent register-tiled FP32 / 4 the fused per-wavenumber stage / 5 the
  * fused stage with D2 v inside it / 6 the fused stage in parity blocks / 7 the
- * same with its float-float D2 v / 8 the register-tiled FP32 stage with its
+ * same with D2 v inside it (on the tensor instructions or in float-float, as in
+ * dns_config) / 8 the register-tiled FP32 stage with its
  * forcing and apply in parity blocks.  Any output may be NULL. */
 int dns_kernel_choice(const dns_handle* h, int group, int* ygemm, int* plane, int* helm);
 

@@ -708,8 +708,8 @@ void cache_store(const char* path, const std::string& key, int choice, const flo
 // config; 0 entries are decided by the autotuner at dns_bind_workspace.
 int choose_variants(dns_handle* h, const dns_config* cfg, GroupView& v, int gi) {
     const dns_group_desc& d = h->descs[gi];
-    // y-contraction variant: 1 register-tiled FP32, 2 tcgen05, 3 register-tiled
-    // FP32 in parity blocks; 0 = decided by the autotuner when the workspace is
+    // y-contraction variant: 1 register-tiled FP32, 2 tcgen05, 3 in parity blocks on
+    // mma.sync; 0 = decided by the autotuner when the workspace is
     // bound (where more than one candidate can run)
     // The tensor-core one accumulates D2 v in FP32, which loses about 1e-5 of
     // |D2 v| to the cancellation in D2's rows at My = 65 (max row sum of |D2_int|
@@ -1365,7 +1365,8 @@ int dns_bind_workspace(dns_handle* h, void* dev_ptr, size_t bytes) {
             choice = 0;
         if (!choice) {
             // timed on sub-step 2 (both accumulators); it writes only the sub-step
-            // state, which set_state overwrites later
+            // state, the forcing terms and their accumulators, which every step
+            // writes before it reads them
             float best[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             // the persistent variant (3) fills the whole GPU, which starves the
             // concurrent groups: only on request.  8: forcing and apply in parity

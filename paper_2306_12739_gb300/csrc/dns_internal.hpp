@@ -21,7 +21,7 @@ struct GroupView {
     int rp;               // Ny rounded up to a multiple of 4 (row padding of transposed operators)
     int kp;               // Ny rounded up to a multiple of 16 (K of the tensor-core y-contraction)
     int ygemm;            // mixed path y-derivatives: 1 register-tiled FP32, 2 tcgen05 split-BF16,
-                          // 3 register-tiled FP32 in parity blocks; 0 = autotune
+                          // 3 in parity blocks on mma.sync (k_spec_mma.cu); 0 = autotune
     int plane;            // plane stage: 1 single-CTA kernel, 2 cluster kernel, 3 line-owned
                           // single-CTA kernel (mixed path), 5 the three-launch split one; 0 = autotune
     const void* Atc;      // tensor-core A image: [D1_int; D2_int] in 3 BF16 pieces

@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_spec(GroupView g, int s) {
 // operators once phase 2 is done (half the products of the natural-order
 // float-float sum).  The D2FF form runs only where the group's fragment images
 // are too large for k_spec_mma.cu (spec_mma_supported), which takes it otherwise:
-// 48 us here against 30 there (64x65x64, 4 members).
+// 48 us here against 32 there (64x65x64, 4 members).
 // ============================================================================
 
 __host__ __device__ inline size_t eo_smem_bytes(const GroupView& g) {

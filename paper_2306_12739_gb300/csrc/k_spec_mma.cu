@@ -858,8 +858,8 @@ size_t spec_mma_smem_bytes(const GroupView& g) {
 }
 
 // Two warps per tile while the chip then still holds every one of them at once (16
-// at 128 registers on each of 152 SMs): 16x33x16 x 1 12.5 us a launch against 17.5,
-// 48x36x32 x 3 15.1 against 19.3; beyond it 64x65x64 x 4 33.1 against 30.5.
+// at 128 registers on each of 152 SMs): 16x33x16 x 1 12.5 us a launch against 16.2,
+// 48x36x32 x 3 16.3 against 19.6; beyond it 64x65x64 x 4 34.2 against 31.5.
 static bool spec_mma_two(const GroupView& g) {
     const long long warps = (long long)(g.npairs - 1) * smm::chunks(g) * smm::tiles(g.ny) *
                             smm::col_tiles(smm::chunk_members(g)) * g.nblk;

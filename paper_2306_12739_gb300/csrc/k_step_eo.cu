@@ -539,9 +539,9 @@ size_t yderiv_eo_smem_bytes(const GroupView& g) {
 bool yderiv_eo_supported(const GroupView& g) { return g.ny >= 3 && yderiv_eo_smem_bytes(g) <= 227 * 1024; }
 
 // On the tensor products (k_spec_mma.cu) wherever D1's and D2's fragments were laid
-// out, which is every group that may take this kernel: 128x97x128 x 4 121.8 -> 76.5
-// us, 64x65x64 x 4 22.8 -> 17.2, 32x97x32 x 4 26.9 -> 11.9, 16x33x16 x 1 10.5 -> 8.8,
-// 32x33x32 x 4 equal (10.4).
+// out, which is every group that may take this kernel: 128x97x128 x 4 121.3 -> 93.3
+// us, 64x65x64 x 4 23.5 -> 19.3, 32x97x32 x 4 27.3 -> 12.7, 32x49x32 x 16 19.1 -> 18.7,
+// 16x33x16 x 1 and 32x33x32 x 4 equal (10.6, 10.8).
 void launch_yderiv_eo(const GroupView& g, const double2* v, const double2* e, cudaStream_t st, int sprev) {
     if (g.D1MM != nullptr && g.D2MM != nullptr) {
         launch_yderiv_mma(g, v, e, st, sprev);
